@@ -268,8 +268,8 @@ sfhk_status sfhk_resample_births(const sfhk_births* pool, int64_t m, int64_t n, 
  * against FP64.
  * The escalation pass runs in FP64 (esc_precision 0: in the planar form
  * without deterministic bins, a kernel that splits each step of 32
- * trajectories over four warps, same arithmetic; otherwise one thread per
- * trajectory), in double-float (esc_precision 1, planar form only; FP64 in the
+ * trajectories, or of 8 with four lanes each where the list is short, over
+ * four warps, same arithmetic; otherwise one thread per trajectory), in double-float (esc_precision 1, planar form only; FP64 in the
  * 3D form), or in FP64 with one thread per trajectory always (esc_precision
  * 2).  Double-float carries ~48 significant bits: on chaotic trajectories its
  * results drift from FP64 (measured: 1.6e-3 in H plateau yields at 1e6
@@ -312,7 +312,10 @@ sfhk_status sfhk_resample_births(const sfhk_births* pool, int64_t m, int64_t n, 
  * arithmetic, det Z = det(in-plane block of Z) * Z_yy) whenever q0x and q0y
  * are NULL; 1 always integrates the full 43-component state.  Endpoints
  * (sfhk_propagate) always use the full state.
- * block: threads per block (0 = library choice, 128; else 64 or 128).
+ * block: threads per block (0 = library choice, 128; else 64 or 128).  An FP64
+ * dipole call in the planar form without deterministic bins runs on the
+ * warp-specialised kernels of the escalation pass when block = chunk_steps = 0
+ * (no scratch), and with one thread per trajectory otherwise.
  * chunk_steps: steps per shared-memory field window (0 = library choice;
  * else a multiple of n_out, 64..8192).
  * ---------------------------------------------------------------------- */

@@ -575,7 +575,9 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
     const size_t esc_b = esc ? align256((size_t)n * 4) : 0;
     const size_t blk_b = esc ? align256((size_t)(compact_blocks(n) + 16) * 4) : 0;
     const size_t state_b = align256((size_t)words * (size_t)n * 4);
-    const size_t rw = redo_scratch_words(n);
+    a.redo_lists = redo_lists();
+    a.quad_limit = quad_limit(target->t.pot, a.redo_lists);
+    const size_t rw = redo_scratch_words(n, a.quad_limit);
     const size_t ctr_b = esc ? (size_t)kSide * rw * 4 : 0;   // redo counters and group plan, per side stream
     const size_t total = part_b + esc_b * (1 + 2 * (size_t)nseg) + blk_b * nseg + (esc ? 256 : 0) + state_b + ctr_b;
     unsigned char* base = nullptr;
@@ -594,7 +596,6 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
     double* amax2 = esc ? reinterpret_cast<double*>(bb + blk_b * nseg + 128) : nullptr;
     uint32_t* state = words ? reinterpret_cast<uint32_t*>(bb + blk_b * nseg + 256) : nullptr;
     int* rctr = esc ? reinterpret_cast<int*>(bb + blk_b * nseg + 256 + state_b) : nullptr;
-    a.redo_lists = redo_lists();
     a.esc_l2 = pp->esc_ratio > 0.0 ? (float)log2(pp->esc_ratio) : 0.f;
     a.esc_l2_big = pp->esc_ratio_big > 0.0 ? (float)log2(pp->esc_ratio_big) : a.esc_l2;
     a.esc_l2_lo = pp->esc_big > 0.0 ? fminf(a.esc_l2, a.esc_l2_big) : a.esc_l2;
@@ -743,7 +744,12 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
         a.esc_bin = esc_bin;
         a.esc_ratio = pp->esc_ratio;
     }
-    st = check_cuda(launch_traj(field->f, target->t, pp->precision, a, s), "trajectory launch");
+    // FP64 planar dipole into atomic bins: the warp-specialised kernels; a caller's own
+    // launch shape (block, chunk_steps) asks for the one-thread-per-trajectory kernel
+    const bool warps64 = mode == 1 && pp->precision == 0 && a.planar && !det && pp->block == 0 && pp->chunk_steps == 0;
+    st = check_cuda(warps64 ? launch_fp64(field->f, target->t, a, s)
+                            : launch_traj(field->f, target->t, pp->precision, a, s),
+                    "trajectory launch");
     if (st) return st;
     if (det) {
         st = check_cuda(launch_reduce_partials(part, n_blocks, field->f.n_bins, d_len, d_vel, s), "reduce launch");

@@ -240,7 +240,7 @@ sfhk_status sfhk_batch_create(int32_t n_cfg, const sfhk_field* const* fields, co
         if (!st) st = check_cuda(cudaMalloc(&b->d_amax2, sizeof(double) * n_cfg), "batch alloc");
         int64_t n_max = 0;
         for (int c = 0; c < n_cfg; ++c) n_max = std::max(n_max, b->n[c]);
-        b->rctr_words = redo_scratch_words(n_max);
+        b->rctr_words = redo_scratch_words(n_max, quad_limit(POT_TONGLIN, redo_lists()));   // the larger limit
         if (!st) st = check_cuda(cudaMalloc(&b->d_rctr, sizeof(int) * 8 * b->rctr_words), "batch alloc");
         for (int c = 0; c < n_cfg && !st; ++c) {
             b->host_cfg[c].a.esc_bin = b->d_esc + b->esc_off[c];
@@ -339,6 +339,7 @@ sfhk_status sfhk_batch_run(sfhk_batch* b, void* stream) {
         e.k_from = b->d_kfrom + b->esc_off[c];
         e.count = b->d_count + c;
         e.redo_lists = redo_lists();
+        e.quad_limit = quad_limit(cfg.t.pot, e.redo_lists);
         e.redo_ctr = b->d_rctr + (size_t)(c % 8) * b->rctr_words;
         st = check_cuda(launch_escalation(cfg.f, cfg.t, b->esc_precision, e, side), "escalation launch");
         if (st) return st;

@@ -1,0 +1,535 @@
+// FP64 planar trajectories with four lanes per trajectory, for short lists.
+//
+// On GB300 a warp's FP64 instruction holds its sub-partition's FP64 unit for 64
+// cycles however many of its 32 lanes are active and however independent the
+// instructions are (measured: 64.1 cycles for chains of 1 to 8 independent FMAs, 1
+// to 32 lanes; 76 with all four sub-partitions busy).  A trajectory's speed is
+// therefore the number of FP64 warp instructions of one step, and a list too short
+// to fill the chip with 32 trajectories a block (redo.cu) runs at the pace of the
+// dynamics warp while most SMs idle.  Here a block of four warps holds 8
+// trajectories and every trajectory has four lanes, which split the work inside a
+// step so that one instruction does four parts of it:
+//   dynamics  lanes = {x', z} x {q, p}: one FMA forms the next stage's positions and
+//             momenta, one chain the RK4 combination of all four; the Tong-Lin
+//             potential's three exponentials are one (lanes 0..2);
+//   matrix    lane s forms stage s's Hessian and action integrand, then lane (i, j)
+//             the entries (i, j) of A, B, C and D;
+//   columns   lane c advances column c, lane k one entry of the out-of-plane block;
+//   bins      lane j forms column j of Z, even lanes the real and odd lanes the
+//             imaginary part of det Z; the GTO terms of an FP64 bin in four parts.
+// FP64 instructions per step: dynamics 84 -> 48 (soft-core), 380 -> 160
+// (Tong-Lin), the whole step 323 -> 135 per 8 trajectories: one block per SM steps
+// 2.1 times as fast as 32 trajectories a block, with 1.7 times the FP64 work per
+// trajectory, so the host and the plan choose by list length (quad_limit).
+//
+// Every value is formed by the same operations in the same order as in TrajP
+// (traj_block.cuh): trajectories, columns, determinants, branches and removals are
+// those of the other FP64 kernels bit for bit; sums over trajectories differ in
+// order.
+#include <algorithm>
+
+#include "redo_warps.cuh"
+#include "sfhk_internal.cuh"
+
+namespace sfhk {
+namespace {
+
+constexpr int kT = kQuadWidth;   // trajectories per block
+constexpr int kThreads = 128;
+// dynamics -> matrix, per stage: q (2), g, aux, p (2), then Tong-Lin: Y, Y1, e2, e4, e6;
+// the stage stride puts lanes of neighbouring stages on different banks
+constexpr int kFields = 12;
+constexpr int kStage = kFields * kT + kT;
+// matrix -> columns: A, B, C, D (4 entries each), the out-of-plane rows (a, b), (c, d), state, S
+constexpr int kM = 16, kState = 20, kAct = 24, kN12 = 25;
+// columns -> bins: columns (4 x 4), out-of-plane (4), state, S
+constexpr int kN23 = 25;
+
+struct QShared {
+    double s01[2][4 * kStage];
+    double s12[2][kN12 * kT];
+    double s23[2][kN23 * kT];
+    double hess[4 * 3 * kT];   // stage Hessians (a, b, c), matrix warp only
+    int alive[kT];             // written by the bins warp, read late by the warps ahead
+};
+
+struct QCommon {
+    int64_t n_first, n_last;   // first and last grid point of the block
+    int n_out;
+    bool have;
+    int64_t i, n0, k_cnt;
+    bool alive0;
+    int t, l;                  // trajectory in the block, lane of the trajectory
+};
+
+__device__ __forceinline__ double from_lane(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+__device__ __forceinline__ double xor_lane(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+
+template <int POT>
+__device__ __forceinline__ PotConst<double> pot_const(const TargetDev& tg) {
+    PotConst<double> pc;
+    pc.a2 = (POT == POT_SOFTCORE || POT == POT_HARMONIC) ? tg.pot_param[0] * tg.pot_param[0] : 0.0;
+    pc.Zc = tg.pot_param[0]; pc.a1 = tg.pot_param[1]; pc.a2t = tg.pot_param[2];
+    pc.a3 = tg.pot_param[3]; pc.a4 = tg.pot_param[4]; pc.a5 = tg.pot_param[5];
+    pc.a6 = tg.pot_param[6];
+    return pc;
+}
+
+// dynamics: the state at grid point n and the stages of the step n -> n + 1.  Lane
+// (component c = l & 1, kind l >> 1): kind 0 carries q_c, kind 1 p_c.
+template <int POT>
+__device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const TrajArgs& a, const QCommon& cm,
+                              QShared& sm) {
+    const PotConst<double> pc = pot_const<POT>(tg);
+    const int t = cm.t, c = cm.l & 1;
+    const bool isp = cm.l >= 2;
+    double b;   // this lane's part of the state
+    {
+        TrajP<double, POT> T;
+        T.init(0.0, 0.0, cm.have ? a.qz[cm.i] : 0.0, cm.have ? a.px[cm.i] : 0.0, cm.have ? a.py[cm.i] : 0.0,
+               cm.have ? a.pz[cm.i] : 0.0);
+        b = isp ? (c ? T.p[2] : T.p[0]) : (c ? T.q[2] : T.q[0]);
+    }
+    const StepK<double> hk = f.k64;
+    const double* E = f.E64;
+    auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(E + j) : 0.0; };
+    double e0 = e_at(2 * cm.n_first), e1 = e_at(2 * cm.n_first + 1), e2 = e_at(2 * cm.n_first + 2);
+    const volatile int* alive = sm.alive;
+    // Tong-Lin: this lane's exponent
+    const double ea = POT == POT_TONGLIN ? -(cm.l == 0 ? pc.a2t : (cm.l == 1 ? pc.a4 : pc.a6)) : 0.0;
+    Producer out(0);
+    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+        const int d = out.acquire();
+        double* const o = sm.s01[d] + t;
+        const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
+        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
+        double y = b, u[4], m3 = 1.0, v3 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            // positions of the stage in every lane; the stage momentum in the q lanes
+            const double x = from_lane(y, t), z = from_lane(y, t + kT);
+            const double pk = from_lane(y, t + (2 + c) * kT);
+            double g, aux = 0.0, Y = 0.0, Y1 = 0.0, ex_l = 0.0;
+            if constexpr (POT == POT_SOFTCORE) {
+                const double r2 = fma(x, x, fma(z, z, pc.a2));
+                const double s = rsq(r2);
+                const double s2 = s * s;
+                g = s2 * s;
+                aux = s;
+            } else if constexpr (POT == POT_TONGLIN) {
+                const double r2 = fma(x, x, z * z);
+                const double ir = rsq(r2);
+                const double r = r2 * ir;
+                ex_l = ex(ea * r);
+                const double x2 = from_lane(ex_l, t), x4 = from_lane(ex_l, t + kT), x6 = from_lane(ex_l, t + 2 * kT);
+                tonglin_y(pc, r, x2, x4, x6, Y, Y1);
+                g = tonglin_g(ir, Y, Y1);
+                aux = ir;
+            } else if constexpr (POT == POT_HARMONIC) {
+                g = pc.a2;
+            } else {
+                g = 0.0;
+            }
+            // -g x' and -(g z + E)
+            const double ek = k == 0 ? e0 : (k == 3 ? e2 : e1);
+            const double kp = -fma(g, c ? z : x, c ? ek : 0.0);
+            u[k] = isp ? kp : pk;
+            double* const os = o + k * kStage;
+            os[cm.l * kT] = isp ? (c ? aux : g) : y;                                    // q_x', q_z, g, aux
+            if constexpr (POT == POT_TONGLIN) {
+                os[(isp ? 4 + c : 6 + c) * kT] = isp ? y : (c ? Y1 : Y);                // p_x', p_z, Y, Y1
+                if (cm.l < 3) os[(8 + cm.l) * kT] = ex_l;
+            } else {
+                if (isp) os[(4 + c) * kT] = y;
+            }
+            if (k < 3) y = fma(k < 2 ? hk.hh : hk.h, u[k], b);
+            else {
+                // the last term of the p_x' combination is -g x' unrounded (so nvcc contracts
+                // it in the other FP64 kernels: found by comparing chaotic trajectories)
+                const bool px = isp && c == 0;
+                m3 = px ? -g : 1.0;
+                v3 = px ? x : u[3];
+            }
+        }
+        // the RK4 combination of this lane's component
+        const double nb = fma(hk.h6, fma(m3, v3, fma(2.0, u[1] + u[2], u[0])), b);
+        if (step) b = nb;
+        out.publish(d);
+        e0 = f0;
+        e1 = f1;
+        e2 = f2;
+    }
+    out.drain();
+}
+
+// matrix: the step matrix of grid point n and the action
+template <int POT>
+__device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommon& cm, QShared& sm) {
+    const PotConst<double> pc = pot_const<POT>(tg);
+    const StepK<double> hk = f.k64;
+    const int t = cm.t, l = cm.l, ei = l >> 1, ej = l & 1;
+    const bool odd = l & 1;
+    const double* E = f.E64;
+    auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(E + j) : 0.0; };
+    const int e_off = l == 0 ? 0 : (l == 3 ? 2 : 1);   // stage l reads E at t, t + h/2, t + h/2, t + h
+    double e_cur = e_at(2 * cm.n_first + e_off);
+    double S = 0.0;
+    Consumer in_q(0);
+    Producer out(1);
+    const double h = hk.h, c2 = hk.c2, c4 = hk.c4, c3 = hk.c3, c1 = hk.h6;
+    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+        const double e_next = e_at(2 * n + 2 + e_off);
+        const int di = in_q.wait();
+        const double* const in = sm.s01[di] + t;
+        // stage l: Hessian data and the action integrand
+        const double* const st = in + l * kStage;
+        const double x = st[0], z = st[kT], g = st[2 * kT], px = st[4 * kT], pz = st[5 * kT];
+        double hs, V;
+        if constexpr (POT == POT_SOFTCORE) {
+            const double s = st[3 * kT], s2 = s * s;
+            hs = -3.0 * g * s2;
+            V = -s;
+        } else if constexpr (POT == POT_TONGLIN) {
+            const double ir = st[3 * kT], Y = st[6 * kT], Y1 = st[7 * kT];
+            const double r = fma(x, x, z * z) * ir;
+            hs = tonglin_h(pc, r, ir, Y, Y1, st[8 * kT], st[9 * kT], st[10 * kT]);
+            V = -Y * ir;
+        } else if constexpr (POT == POT_HARMONIC) {
+            hs = 0.0;
+            V = 0.5 * pc.a2 * fma(x, x, z * z);
+        } else {
+            hs = 0.0;
+            V = 0.0;
+        }
+        const double hx = hs * x;
+        double* const H = sm.hess + t;
+        H[(3 * l) * kT] = fma(hx, x, g);
+        H[(3 * l + 1) * kT] = hx * z;
+        H[(3 * l + 2) * kT] = fma(hs * z, z, g);
+        const double kS = TrajP<double, POT>::action_term(px, pz, z, e_cur, V);
+        const double g0 = in[2 * kT], g1 = in[kStage + 2 * kT], g2 = in[2 * kStage + 2 * kT],
+                     g3 = in[3 * kStage + 2 * kT];
+        const double state_l = in[(l < 2 ? l : l + 2) * kT];   // q_x', q_z, p_x', p_z at n
+        in_q.release(di);
+        __syncwarp();
+        const int dq = out.acquire();
+        double* const o = sm.s12[dq] + t;
+        // entry (ei, ej) from row ei of H3, H4 and column ej of H1, H2
+        auto He = [&](int s, int i, int j) { return H[(3 * s + i + j) * kT]; };
+        const double h0e = He(0, ei, ej), h1e = He(1, ei, ej), h2e = He(2, ei, ej), h3e = He(3, ei, ej);
+        const double p31 = fma(He(2, ei, 0), He(0, 0, ej), He(2, ei, 1) * He(0, 1, ej));
+        const double p42 = fma(He(3, ei, 0), He(1, 0, ej), He(3, ei, 1) * He(1, 1, ej));
+        __syncwarp();   // the Hessians are read before the next grid point writes them
+        const double s23 = h1e + h2e;
+        o[l * kT] = fma(c4, p31, -c2 * (s23 + h0e));
+        o[(4 + l) * kT] = fma(-c3, s23, ei == ej ? h : 0.0);
+        o[(8 + l) * kT] = fma(c3, p31 + p42, -c1 * (fma(2.0, s23, h0e) + h3e));
+        o[(12 + l) * kT] = fma(c4, p42, -c2 * (s23 + h3e));
+        // out-of-plane rows: (a, b) in even lanes, (c, d) in odd lanes
+        const double g23 = g1 + g2;
+        const double ad = fma(c4, (odd ? g3 : g2) * (odd ? g1 : g0), -c2 * (g23 + (odd ? g3 : g0)));
+        const double w = fma(g2, g0, g3 * g1), v = -c1 * (fma(2.0, g23, g0) + g3);
+        const double bc = fma(odd ? c3 : -c3, odd ? w : g23, odd ? v : h);
+        if (l < 2) {
+            o[(kM + 2 * l) * kT] = odd ? bc : ad;
+            o[(kM + 2 * l + 1) * kT] = odd ? ad : bc;
+        }
+        o[(kState + l) * kT] = state_l;
+        if (l == 0) o[kAct * kT] = S;   // the action at grid point n
+        // h/6 (k1 + 2 (k2 + k3) + k4)
+        const double k1 = from_lane(kS, t), k2 = from_lane(kS, t + kT), k3 = from_lane(kS, t + 2 * kT),
+                     k4 = from_lane(kS, t + 3 * kT);
+        if (cm.have && n >= cm.n0 && n < cm.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, c1);
+        out.publish(dq);
+        e_cur = e_next;
+    }
+    out.drain();
+}
+
+// columns: lane c advances column c of the in-plane block; lanes 0..3 hold
+// dy/dy0, dpy/dy0, dy/dpy0, dpy/dpy0 of the out-of-plane block
+__device__ void quad_columns(const QCommon& cm, QShared& sm) {
+    const int t = cm.t, l = cm.l;
+    const bool odd = l & 1;
+    double X0 = l == 0 ? 1.0 : 0.0, X1 = l == 1 ? 1.0 : 0.0, Y0 = l == 2 ? 1.0 : 0.0, Y1 = l == 3 ? 1.0 : 0.0;
+    double w = (l == 0 || l == 3) ? 1.0 : 0.0;
+    const volatile int* alive = sm.alive;
+    Consumer in_q(1);
+    Producer out(2);
+    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+        const int di = in_q.wait();
+        const double* const in = sm.s12[di] + t;
+        const double wp = xor_lane(w, kT);   // the other entry of this out-of-plane column
+        if (cm.have && n >= cm.n0 && n < cm.n_last && alive[t]) {
+            const double x0 = X0, x1 = X1, y0 = Y0, y1 = Y1;
+            X0 = fma(in[0], x0, fma(in[kT], x1, fma(in[4 * kT], y0, fma(in[5 * kT], y1, x0))));
+            X1 = fma(in[2 * kT], x0, fma(in[3 * kT], x1, fma(in[5 * kT], y0, fma(in[7 * kT], y1, x1))));
+            Y0 = fma(in[8 * kT], x0, fma(in[9 * kT], x1, fma(in[12 * kT], y0, fma(in[13 * kT], y1, y0))));
+            Y1 = fma(in[10 * kT], x0, fma(in[11 * kT], x1, fma(in[14 * kT], y0, fma(in[15 * kT], y1, y1))));
+            const double m0 = in[(kM + 2 * odd) * kT], m1 = in[(kM + 2 * odd + 1) * kT];
+            const double q = odd ? wp : w, p = odd ? w : wp;
+            w = fma(m0, q, fma(m1, p, w));
+        }
+        const double state_l = in[(kState + l) * kT];
+        const double S = in[kAct * kT];
+        in_q.release(di);
+        const int dq = out.acquire();
+        double* const o = sm.s23[dq] + t;
+        o[(4 * l) * kT] = X0;
+        o[(4 * l + 1) * kT] = X1;
+        o[(4 * l + 2) * kT] = Y0;
+        o[(4 * l + 3) * kT] = Y1;
+        o[(16 + l) * kT] = w;
+        o[(20 + l) * kT] = state_l;
+        if (l == 0) o[24 * kT] = S;
+        out.publish(dq);
+    }
+    out.drain();
+}
+
+// bins: det Z and its branch, labels, removal, prefactor and the recombination sums
+template <int POT>
+__device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms& gt, const TrajArgs& a,
+                          const QCommon& c, QShared& sm) {
+    const int t = c.t, l = c.l;
+    const bool odd = l & 1;
+    const Cx<double> amp{c.have ? a.amp_re[c.i] : 0.0, c.have ? a.amp_im[c.i] : 0.0};
+    const bool fbins = a.float_bins != 0;   // recombination terms in float (as the float pass forms them)
+    const float gamf = (float)a.gamma;
+    bool alive = c.alive0;
+    unsigned flags = (c.have && !alive) ? 8u : 0u;
+    Cx2<double> Dp{1.0, 0.0};
+    double sgn = 1.0;
+    const double hz = 0.5, gz = -a.gamma, qz = a.qg64;
+    const bool pw = a.pw_mask != 0;
+    const double pw_r2 = a.pw_radius * a.pw_radius;
+    int pw_cls = -1;
+    bool pw_in = false;
+    unsigned long long all_steps = 0, steps = 0;
+    int rem = (int)(c.n_first % c.n_out);
+    int64_t k_bin = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
+    volatile int* alive_out = sm.alive;
+    Consumer in_q(2);
+    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+        const int di = in_q.wait();
+        const double* const in = sm.s23[di] + t;
+        const double X0 = in[(4 * l) * kT], X1 = in[(4 * l + 1) * kT], Y0 = in[(4 * l + 2) * kT],
+                     Y1 = in[(4 * l + 3) * kT];
+        const double aq = in[16 * kT], ap = in[17 * kT], bq = in[18 * kT], bp = in[19 * kT];
+        const double q0 = in[20 * kT], q2 = in[21 * kT], p0 = in[22 * kT], p2 = in[23 * kT], S = in[24 * kT];
+        in_q.release(di);
+        const bool on_bin = rem == 0;
+        // partial waves (Sec. III.A-B), as in redo.cu
+        if (pw && alive && n >= c.n0) {
+            const double qx = q0, qy = 0.0, qzz = q2;
+            const bool inside = qx * qx + qy * qy + qzz * qzz < pw_r2;
+            if (inside && !pw_in) {
+                const double px = p0, py = 0.0, pz = p2;
+                const double lx = qy * pz - qzz * py, ly = qzz * px - qx * pz, lz = qx * py - qy * px;
+                const double L2 = lx * lx + ly * ly + lz * lz;
+                pw_cls = L2 < 0.25 ? 0 : (L2 < 2.25 ? 1 : (L2 < 6.25 ? 2 : 3));
+            }
+            pw_in = inside;
+        }
+        const bool pw_ok = !pw || (pw_cls >= 0 && ((a.pw_mask >> pw_cls) & 1));
+        if (on_bin) {
+            bool valid = false;
+            Cx<double> C{0.0, 0.0};
+            if (alive && n >= c.n0) {
+                const double fs = q0 + q2 + p0 + p2;
+                const bool ok = isfinite(fs) && isfinite(S);
+                const cd D{Dp.re, Dp.im};
+                const double m2 = D.re * D.re + D.im * D.im;
+                if (!ok || !(m2 <= a.d_t * a.d_t)) {
+                    alive = false;
+                    flags |= 1u;
+                    if (!ok || !isfinite(m2)) flags |= 2u;
+                } else if (n >= c.k_cnt && pw_ok) {
+                    cd Cz = c_sqrt(D);
+                    if (sgn < 0.0) Cz = -Cz;
+                    C = Cx<double>{Cz.re, Cz.im};
+                    valid = true;
+                }
+            }
+            if (__any_sync(0xffffffffu, valid)) {
+                const double tk = f.t_start + (double)n * f.dt;
+                double sn, cs, cl = 0.0, cv = 0.0;
+                sincos(fmod(tg.ip * tk, 2.0 * kPi), &sn, &cs);
+                if (fbins) {
+                    if (valid && l == 0) {
+                        const FloatState fsn(q0, 0.0, q2, p0, 0.0, p2, S);
+                        float fl, fv;
+                        contribution<float>(fsn, gt, gamf, Cx<float>{(float)C.re, (float)C.im},
+                                            Cx<float>{(float)amp.re, (float)amp.im}, Cx<float>{(float)cs, (float)(-sn)},
+                                            fl, fv);
+                        cl = (double)fl;
+                        cv = (double)fv;
+                    }
+                } else {
+                    // the GTO terms in four parts
+                    const PView v(q0, q2, p0, p2, S);
+                    double pp, qq, pq;
+                    recomb_invariants<double>(v, pp, qq, pq);
+                    GtoSums<double> g{};
+                    if (valid)
+                        for (int j = l; j < gt.n; j += 4) gto_terms<double>(gt, pp, qq, pq, j, j + 1, g);
+                    auto fold = [](double& x) {
+                        x += xor_lane(x, kT);
+                        x += xor_lane(x, 2 * kT);
+                    };
+                    fold(g.s0.re);
+                    fold(g.s0.im);
+                    fold(g.s1.re);
+                    fold(g.s1.im);
+                    if (gt.l == 1) {
+                        fold(g.s2.re);
+                        fold(g.s2.im);
+                        fold(g.s3.re);
+                        fold(g.s3.im);
+                    }
+                    if (valid && l == 0)
+                        contribution_final<double>(v, gt, a.gamma, C, amp, Cx<double>{cs, -sn}, g, cl, cv);
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {   // over the trajectories (lanes 0..7 hold them)
+                    cl += xor_lane(cl, o);
+                    cv += xor_lane(cv, o);
+                }
+                if ((threadIdx.x & 31) == 0 && k_bin < f.n_bins && (cl != 0.0 || cv != 0.0)) {
+                    atomicAdd(&a.d_len[k_bin], cl);
+                    atomicAdd(&a.d_vel[k_bin], cv);
+                }
+            }
+            ++k_bin;
+        }
+        alive_out[t] = alive ? 1 : 0;
+        rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
+        // the step n -> n + 1: det Z of the advanced columns (TrajP::detc in parts)
+        const double X0p = xor_lane(X0, 2 * kT), X1p = xor_lane(X1, 2 * kT), Y0p = xor_lane(Y0, 2 * kT),
+                     Y1p = xor_lane(Y1, 2 * kT);   // column l + 2 in lanes 0 and 1
+        double zr0 = hz * (Y0p + X0), zr1 = hz * (Y1p + X1);
+        double zi0 = fma(gz, X0p, qz * Y0), zi1 = fma(gz, X1p, qz * Y1);
+        // column (l & 1) of Z in every lane, then both
+        zr0 = from_lane(zr0, t + odd * kT);
+        zr1 = from_lane(zr1, t + odd * kT);
+        zi0 = from_lane(zi0, t + odd * kT);
+        zi1 = from_lane(zi1, t + odd * kT);
+        const double wr0 = xor_lane(zr0, kT), wr1 = xor_lane(zr1, kT), wi0 = xor_lane(zi0, kT), wi1 = xor_lane(zi1, kT);
+        const double r00 = odd ? wr0 : zr0, r10 = odd ? wr1 : zr1, i00 = odd ? wi0 : zi0, i10 = odd ? wi1 : zi1;
+        const double r01 = odd ? zr0 : wr0, r11 = odd ? zr1 : wr1, i01 = odd ? zi0 : wi0, i11 = odd ? zi1 : wi1;
+        const double u1 = i00 * (odd ? r11 : i11), u2 = i01 * (odd ? r10 : i10);
+        const double dd = fma(r00, odd ? i11 : r11, odd ? u1 : -u1) - fma(r01, odd ? i10 : r10, odd ? u2 : -u2);
+        const double dx = xor_lane(dd, kT);
+        const double ar = odd ? dx : dd, ai = odd ? dd : dx;
+        const double yr = hz * (bp + aq), yi = fma(gz, bq, qz * ap);
+        const double u3 = ai * (odd ? yr : yi);
+        const double de = fma(ar, odd ? yi : yr, odd ? u3 : -u3);
+        const double df = xor_lane(de, kT);
+        if (alive && n >= c.n0 && n < c.n_last) {
+            follow_branch<double>(Dp, Cx2<double>{odd ? df : de, odd ? de : df}, sgn, flags);
+            ++all_steps;
+            if (n >= c.k_cnt) ++steps;
+        }
+    }
+    if (a.stats) {
+        const bool one = l == 0;   // a trajectory is counted by its first lane
+        unsigned rm = __reduce_add_sync(0xffffffffu, one && (flags & 1u) ? 1u : 0u);
+        unsigned nf = __reduce_add_sync(0xffffffffu, one && (flags & 2u) ? 1u : 0u);
+        unsigned bg = __reduce_add_sync(0xffffffffu, one && (flags & 4u) ? 1u : 0u);
+        unsigned sk = __reduce_add_sync(0xffffffffu, one && (flags & 8u) ? 1u : 0u);
+        unsigned long long st = one ? steps : 0, ast = one ? all_steps : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            st += __shfl_xor_sync(0xffffffffu, st, o);
+            ast += __shfl_xor_sync(0xffffffffu, ast, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            if (rm) atomicAdd(&a.stats->removed, (unsigned long long)rm);
+            if (nf) atomicAdd(&a.stats->nonfinite, (unsigned long long)nf);
+            if (bg) atomicAdd(&a.stats->branch_guard, (unsigned long long)bg);
+            if (sk) atomicAdd(&a.stats->skipped, (unsigned long long)sk);
+            if (a.idx && ast) atomicAdd(&a.stats->esc_steps, ast);
+            if (a.idx && ast > st) atomicAdd(&a.stats->esc_steps_pre, ast - st);
+            if (st) atomicAdd(&a.stats->traj_steps, st);
+        }
+    }
+}
+
+// One group of 8 list entries (list positions 8 g .. 8 g + 7).
+template <int POT>
+__device__ void quad_group(const FieldDev& f, const TargetDev& tg, const GtoTerms& gt, const TrajArgs& a, int64_t g,
+                           int64_t n_list, QShared& sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    QCommon c;
+    c.t = lane & (kT - 1);
+    c.l = lane / kT;
+    c.n_out = (int)f.n_out;
+    c.n_last = a.n_last;
+    const int64_t j = g * kT + c.t;
+    c.have = j < n_list;
+    c.i = c.have ? (a.idx ? (int64_t)a.idx[j] : j) : 0;
+    c.k_cnt = (c.have && a.k_from) ? (int64_t)a.k_from[j] * c.n_out : 0;
+    c.n0 = c.have ? (int64_t)a.n0[c.i] : 0;
+    const double ar = c.have ? a.amp_re[c.i] : 0.0, ai = c.have ? a.amp_im[c.i] : 0.0;
+    c.alive0 = c.have && c.n0 <= a.n_last && c.n0 >= 0 && (ar != 0.0 || ai != 0.0);
+    long long m = c.alive0 ? (long long)c.n0 : LLONG_MAX;   // first grid point of the block
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const long long u = __shfl_xor_sync(0xffffffffu, m, o);
+        m = u < m ? u : m;
+    }
+    if (m == LLONG_MAX) {
+        // nothing to integrate; one warp still reports skipped births
+        if (a.stats && warp == 0) {
+            const unsigned sk = __reduce_add_sync(0xffffffffu, c.have && c.l == 0 ? 1u : 0u);
+            if (lane == 0 && sk) atomicAdd(&a.stats->skipped, (unsigned long long)sk);
+        }
+        return;
+    }
+    c.n_first = m;
+    if (warp == 0 && c.l == 0) sm.alive[c.t] = c.alive0 ? 1 : 0;
+    __syncthreads();
+    const int role = (warp + (int)(g & 3)) & 3;
+    if (role == 0) quad_dynamics<POT>(f, tg, a, c, sm);
+    else if (role == 1) quad_matrix<POT>(f, tg, c, sm);
+    else if (role == 2) quad_columns(c, sm);
+    else quad_bins<POT>(f, tg, gt, a, c, sm);
+}
+
+template <int POT>
+__global__ void __launch_bounds__(kThreads, 3) quad_kernel(FieldDev f, TargetDev tg, GtoTerms gt, TrajArgs a) {
+    __shared__ QShared sm;
+    __shared__ long long s_g;
+    const int64_t n_list = a.count ? (int64_t)*a.count : a.n;
+    if (a.count && n_list > a.quad_limit) return;   // a long list: redo.cu takes it
+    GroupSource src(a, (n_list + kT - 1) / kT);
+    for (;;) {
+        const int64_t g = src.next(a, s_g);
+        if (g < 0) break;
+        quad_group<POT>(f, tg, gt, a, g, n_list, sm);
+        __syncthreads();   // every role has drained its hand-offs before the next group
+    }
+}
+
+template <int POT>
+cudaError_t launch_pot(const FieldDev& f, const TargetDev& t, const GtoTerms& gt, const TrajArgs& a, cudaStream_t s) {
+    const int64_t most = std::min<int64_t>(a.n, a.count ? a.quad_limit : a.n);
+    const int64_t need = (most + kT - 1) / kT;
+    const int64_t blocks = a.redo_ctr ? std::min<int64_t>(need, (int64_t)a.redo_lists * 4) : need;
+    quad_kernel<POT><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_quad(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
+    const GtoTerms gt = make_gto_terms(t, a.gamma);
+    switch (t.pot) {
+        case POT_SOFTCORE: return launch_pot<POT_SOFTCORE>(f, t, gt, a, s);
+        case POT_TONGLIN: return launch_pot<POT_TONGLIN>(f, t, gt, a, s);
+        case POT_HARMONIC: return launch_pot<POT_HARMONIC>(f, t, gt, a, s);
+        default: return launch_pot<POT_ZERO>(f, t, gt, a, s);
+    }
+}
+
+}  // namespace sfhk

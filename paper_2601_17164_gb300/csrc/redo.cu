@@ -35,8 +35,8 @@
 // four) differs.
 #include <algorithm>
 
+#include "redo_warps.cuh"
 #include "sfhk_internal.cuh"
-#include "traj_block.cuh"
 
 namespace sfhk {
 namespace {
@@ -52,55 +52,6 @@ constexpr int kS01 = 33;
 // within 48 KB per block)
 constexpr int kS12 = 36;
 constexpr int kS23 = 25;          // columns -> bins: columns after the step (16 in-plane, 4 out-of-plane), state
-
-// read-only view of the planar state for the recombination terms (q_y = p_y = 0)
-struct PView {
-    double q[3], p[3];
-    struct {
-        double s;
-        __device__ double reduced() const { return s; }
-    } S;
-    __device__ PView(double q0, double q2, double p0, double p2, double s) : q{q0, 0.0, q2}, p{p0, 0.0, p2}, S{s} {}
-};
-
-// Two-slot hand-offs between consecutive roles on named barriers (0 is left to
-// __syncthreads): hand-off h in {0, 1, 2}, slot d in {0, 1}; "full" is arrived at by
-// the producer and waited on by the consumer, "empty" the other way round, 64
-// threads each (the two warps).  A role runs ahead of the next by at most two
-// grid points, so uneven work per grid point evens out across the pipeline.
-__device__ __forceinline__ void bar_sync64(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
-__device__ __forceinline__ void bar_arrive64(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
-struct Producer {
-    int h;
-    int64_t k;
-    __device__ explicit Producer(int h_) : h(h_), k(0) {}
-    __device__ int acquire() {                     // slot for item k, once its item k - 2 is consumed
-        const int d = (int)(k & 1);
-        if (k >= 2) bar_sync64(3 + 4 * h + d);
-        return d;
-    }
-    __device__ void publish(int d) {
-        bar_arrive64(1 + 4 * h + d);
-        ++k;
-    }
-    __device__ void drain() {                      // the consumer's releases of the last items
-        for (int64_t j = (k >= 2 ? k - 2 : 0); j < k; ++j) bar_sync64(3 + 4 * h + (int)(j & 1));
-    }
-};
-struct Consumer {
-    int h;
-    int64_t k;
-    __device__ explicit Consumer(int h_) : h(h_), k(0) {}
-    __device__ int wait() {
-        const int d = (int)(k & 1);
-        bar_sync64(1 + 4 * h + d);
-        return d;
-    }
-    __device__ void release(int d) {
-        bar_arrive64(3 + 4 * h + d);
-        ++k;
-    }
-};
 
 struct Shared {
     double s01[2][kS01][kW];
@@ -454,8 +405,8 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
             if (nf) atomicAdd(&a.stats->nonfinite, (unsigned long long)nf);
             if (bg) atomicAdd(&a.stats->branch_guard, (unsigned long long)bg);
             if (sk) atomicAdd(&a.stats->skipped, (unsigned long long)sk);
-            if (ast) atomicAdd(&a.stats->esc_steps, ast);
-            if (ast > st) atomicAdd(&a.stats->esc_steps_pre, ast - st);
+            if (a.idx && ast) atomicAdd(&a.stats->esc_steps, ast);
+            if (a.idx && ast > st) atomicAdd(&a.stats->esc_steps_pre, ast - st);
             if (st) atomicAdd(&a.stats->traj_steps, st);
         }
     }
@@ -470,8 +421,8 @@ __device__ void redo_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     c.n_last = a.n_last;
     const int64_t j = g * kW + lane;
     c.have = j < n_list;
-    c.i = c.have ? (int64_t)a.idx[j] : 0;
-    const int64_t k_min = c.have ? (int64_t)a.k_from[j] : 0;
+    c.i = c.have ? (a.idx ? (int64_t)a.idx[j] : j) : 0;
+    const int64_t k_min = (c.have && a.k_from) ? (int64_t)a.k_from[j] : 0;
     c.k_cnt = k_min * c.n_out;
     c.n0 = c.have ? (int64_t)a.n0[c.i] : 0;
     const double ar = c.have ? a.amp_re[c.i] : 0.0, ai = c.have ? a.amp_im[c.i] : 0.0;
@@ -501,12 +452,6 @@ __device__ void redo_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     else run_bins<POT>(f, tg, gt, a, c, sm, lane);
 }
 
-__device__ __forceinline__ unsigned sm_id() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
-    return r;
-}
-
 // Groups to SMs.  The list is in birth order, so group g's length (grid points from
 // its earliest birth to the end) falls with g.  One warp plans the launch: it takes
 // the groups longest first and gives each to the list (one per SM) with the least
@@ -518,7 +463,8 @@ __device__ __forceinline__ unsigned sm_id() {
 // every group is taken exactly once whatever the SMs' numbering and the blocks'
 // placement.
 __global__ void redo_plan_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ n0,
-                                 const int32_t* __restrict__ count, int64_t n_last, int L, int64_t g_max, int* plan) {
+                                 const int32_t* __restrict__ count, int64_t n_last, int L, int64_t quad_limit, int64_t g_max,
+                                 int* plan) {
     __shared__ long long load[kRedoLists];
     __shared__ int cursor[kRedoLists];
     const int lane = threadIdx.x;   // one warp
@@ -527,7 +473,8 @@ __global__ void redo_plan_kernel(const int32_t* __restrict__ idx, const int32_t*
     int* const grp = plan + 3 * kRedoLists;
     int* const asg = grp + g_max;
     const int64_t n_list = *count;
-    const int64_t G = min((n_list + kW - 1) / kW, g_max);
+    const int W = n_list <= quad_limit ? kQuadWidth : kW;   // trajectories per group
+    const int64_t G = min((n_list + W - 1) / W, g_max);
     for (int l = lane; l < L; l += 32) {
         load[l] = 0;
         cursor[l] = 0;
@@ -535,9 +482,9 @@ __global__ void redo_plan_kernel(const int32_t* __restrict__ idx, const int32_t*
     __syncwarp();
     for (int64_t g = 0; g < G; ++g) {
         // the group's length: from its earliest birth in range to the end
-        const int64_t j = g * kW + lane;
+        const int64_t j = g * W + lane;
         long long m = LLONG_MAX;
-        if (j < n_list) {
+        if (lane < W && j < n_list) {
             const long long b = n0[idx[j]];
             if (b >= 0 && b <= n_last) m = b;
         }
@@ -590,26 +537,14 @@ __global__ void __launch_bounds__(kThreads, 4) redo_kernel(FieldDev f, TargetDev
     __shared__ Shared sm;
     __shared__ long long s_g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t n_list = (int64_t)*a.count;
-    const int L = a.redo_lists;
-    const int* const len = a.redo_ctr + kRedoLists;
-    const int* const start = a.redo_ctr + 2 * kRedoLists;
-    const int* const grp = a.redo_ctr + 3 * kRedoLists;
-    const int home = (int)(sm_id() % (unsigned)L);
-    for (int probe = 0; probe < L; ++probe) {
-        const int l = (home + probe) % L;
-        for (;;) {
-            if (threadIdx.x == 0) {
-                const int k = atomicAdd(&a.redo_ctr[l], 1);
-                s_g = k < len[l] ? (long long)grp[start[l] + k] : -1;
-            }
-            __syncthreads();
-            const long long g = s_g;
-            __syncthreads();   // every thread has read s_g before thread 0 writes the next
-            if (g < 0) break;
-            redo_group<POT>(f, tg, gt, a, (int64_t)g, n_list, sm, lane, warp);
-            __syncthreads();   // every role has drained its hand-offs before the next group
-        }
+    const int64_t n_list = a.count ? (int64_t)*a.count : a.n;
+    if (a.count && n_list <= a.quad_limit) return;   // a short list: quad.cu takes it
+    GroupSource src(a, (n_list + kW - 1) / kW);
+    for (;;) {
+        const int64_t g = src.next(a, s_g);
+        if (g < 0) break;
+        redo_group<POT>(f, tg, gt, a, g, n_list, sm, lane, warp);
+        __syncthreads();   // every role has drained its hand-offs before the next group
     }
 }
 
@@ -617,9 +552,19 @@ template <int POT>
 cudaError_t launch_pot(const FieldDev& f, const TargetDev& t, const GtoTerms& gt, const TrajArgs& a, cudaStream_t s) {
     // persistent: as many blocks as fit (4 per SM), each looping over groups
     const int64_t need = (a.n + kW - 1) / kW;   // an upper bound on the groups (the count is on the device)
-    const int64_t blocks = std::min<int64_t>(need, (int64_t)a.redo_lists * 4);
+    const int64_t blocks = a.redo_ctr ? std::min<int64_t>(need, (int64_t)a.redo_lists * 4) : need;
     redo_kernel<POT><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
     return cudaGetLastError();
+}
+
+cudaError_t launch_wide(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
+    const GtoTerms gt = make_gto_terms(t, a.gamma);
+    switch (t.pot) {
+        case POT_SOFTCORE: return launch_pot<POT_SOFTCORE>(f, t, gt, a, s);
+        case POT_TONGLIN: return launch_pot<POT_TONGLIN>(f, t, gt, a, s);
+        case POT_HARMONIC: return launch_pot<POT_HARMONIC>(f, t, gt, a, s);
+        default: return launch_pot<POT_ZERO>(f, t, gt, a, s);
+    }
 }
 
 }  // namespace
@@ -633,23 +578,33 @@ int redo_lists() {
     return std::max(1, std::min(sms, kRedoLists));
 }
 
+// Longest list for the four-lane kernel, from FP64 instructions per step (64 cycles on
+// the longest role, 19 per SM for all roles): with m groups of 8 per SM it steps in
+// max(48 x 64, m x 135 x 19) cycles (soft-core), the 32-wide kernel with one group
+// per SM in about 7,600: two groups of 8 per SM win, three do not.  Tong-Lin: max(160
+// x 64, m x 265 x 19) against 24,000: four do.
+int64_t quad_limit(int pot, int lists) { return (int64_t)kQuadWidth * lists * (pot == POT_TONGLIN ? 4 : 2); }
+
+cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
+    if (a.n == 0) return cudaSuccess;
+    if (a.redo_lists < 1 || a.redo_lists > kRedoLists) return cudaErrorInvalidValue;
+    if (a.n <= a.quad_limit) return launch_quad(f, t, a, s);
+    return launch_wide(f, t, a, s);
+}
+
 cudaError_t launch_redo(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     if (a.redo_lists < 1 || a.redo_ctr == nullptr) return cudaErrorInvalidValue;
     if (a.redo_lists > kRedoLists) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(a.redo_ctr, 0, (size_t)a.redo_lists * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    redo_plan_kernel<<<1, 32, 0, s>>>(a.idx, a.n0, a.count, a.n_last, a.redo_lists, (int64_t)((a.n + kW - 1) / kW + 1),
-                                      a.redo_ctr);
+    redo_plan_kernel<<<1, 32, 0, s>>>(a.idx, a.n0, a.count, a.n_last, a.redo_lists, a.quad_limit,
+                                      redo_groups(a.n, a.quad_limit), a.redo_ctr);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const GtoTerms gt = make_gto_terms(t, a.gamma);
-    switch (t.pot) {
-        case POT_SOFTCORE: return launch_pot<POT_SOFTCORE>(f, t, gt, a, s);
-        case POT_TONGLIN: return launch_pot<POT_TONGLIN>(f, t, gt, a, s);
-        case POT_HARMONIC: return launch_pot<POT_HARMONIC>(f, t, gt, a, s);
-        default: return launch_pot<POT_ZERO>(f, t, gt, a, s);
-    }
+    // the list's length is on the device: the kernel that it is not meant for returns at once
+    if (e == cudaSuccess && a.quad_limit > 0) e = launch_quad(f, t, a, s);
+    if (e == cudaSuccess && a.n > a.quad_limit) e = launch_wide(f, t, a, s);
+    return e;
 }
 
 }  // namespace sfhk

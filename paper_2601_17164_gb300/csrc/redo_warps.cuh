@@ -1,0 +1,118 @@
+// Pieces shared by the warp-specialised FP64 kernels (redo.cu, quad.cu): the hand-off
+// rings between the warps of a block, the view of a planar state that the
+// recombination terms take, and the SM id.
+#pragma once
+
+#include "traj_block.cuh"
+
+namespace sfhk {
+namespace {
+
+// read-only view of the planar state for the recombination terms (q_y = p_y = 0)
+struct PView {
+    double q[3], p[3];
+    struct {
+        double s;
+        __device__ double reduced() const { return s; }
+    } S;
+    __device__ PView(double q0, double q2, double p0, double p2, double s) : q{q0, 0.0, q2}, p{p0, 0.0, p2}, S{s} {}
+};
+
+// Two-slot hand-offs between consecutive roles on named barriers (0 is left to
+// __syncthreads): hand-off h in {0, 1, 2}, slot d in {0, 1}; "full" is arrived at by
+// the producer and waited on by the consumer, "empty" the other way round, 64
+// threads each (the two warps).  A role runs ahead of the next by at most two
+// grid points, so uneven work per grid point evens out across the pipeline.
+// The barrier instructions want the warp converged.
+__device__ __forceinline__ void bar_sync64(int id) {
+    __syncwarp();
+    asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void bar_arrive64(int id) {
+    __syncwarp();
+    asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory");
+}
+struct Producer {
+    int h;
+    int64_t k;
+    __device__ explicit Producer(int h_) : h(h_), k(0) {}
+    __device__ int acquire() {                     // slot for item k, once its item k - 2 is consumed
+        const int d = (int)(k & 1);
+        if (k >= 2) bar_sync64(3 + 4 * h + d);
+        return d;
+    }
+    __device__ void publish(int d) {
+        bar_arrive64(1 + 4 * h + d);
+        ++k;
+    }
+    __device__ void drain() {                      // the consumer's releases of the last items
+        for (int64_t j = (k >= 2 ? k - 2 : 0); j < k; ++j) bar_sync64(3 + 4 * h + (int)(j & 1));
+    }
+};
+struct Consumer {
+    int h;
+    int64_t k;
+    __device__ explicit Consumer(int h_) : h(h_), k(0) {}
+    __device__ int wait() {
+        const int d = (int)(k & 1);
+        bar_sync64(1 + 4 * h + d);
+        return d;
+    }
+    __device__ void release(int d) {
+        bar_arrive64(3 + 4 * h + d);
+        ++k;
+    }
+};
+
+__device__ __forceinline__ unsigned sm_id() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
+    return r;
+}
+
+// Where a block's next group of list entries comes from.  With a plan (redo_plan_kernel):
+// the groups of its own SM's list, longest first, then those left on the other lists,
+// one atomic counter per list.  Without one (a call that must not touch the shared
+// scratch): one group per block, rows of L blocks taken in alternating direction so
+// that a column of blocks (about one SM's) gets long and short groups.
+struct GroupSource {
+    int probe, home;
+    int64_t g_static;
+    __device__ GroupSource(const TrajArgs& a, int64_t n_groups) : probe(0), home(0), g_static(-1) {
+        const int L = a.redo_lists;
+        if (a.redo_ctr) {
+            home = (int)(sm_id() % (unsigned)L);
+        } else {
+            const int64_t b = blockIdx.x, row = b / L, pos = b - row * L;
+            const int64_t len = n_groups - row * L < L ? n_groups - row * L : L;
+            if (pos < len) g_static = row * L + ((row & 1) ? len - 1 - pos : pos);
+        }
+    }
+    // the next group, -1 when none is left; called by every thread of the block
+    __device__ int64_t next(const TrajArgs& a, long long& s_g) {
+        if (!a.redo_ctr) {
+            const int64_t g = g_static;
+            g_static = -1;
+            return g;
+        }
+        const int L = a.redo_lists;
+        const int* const len = a.redo_ctr + kRedoLists;
+        const int* const start = a.redo_ctr + 2 * kRedoLists;
+        const int* const grp = a.redo_ctr + 3 * kRedoLists;
+        for (; probe < L; ++probe) {
+            const int l = (home + probe) % L;
+            if (threadIdx.x == 0) {
+                const int k = atomicAdd(&a.redo_ctr[l], 1);
+                s_g = k < len[l] ? (long long)grp[start[l] + k] : -1;
+            }
+            __syncthreads();
+            const long long g = s_g;
+            __syncthreads();   // every thread has read s_g before thread 0 writes the next
+            if (g >= 0) return g;
+        }
+        return -1;
+    }
+};
+
+}  // namespace
+}  // namespace sfhk

@@ -168,6 +168,7 @@ struct TrajArgs {
     // clears them), then the plan that assigns the list's groups to the lists
     int redo_lists;
     int* redo_ctr;
+    int64_t quad_limit;   // lists up to this length run with four lanes per trajectory (quad.cu)
 };
 cudaError_t launch_traj(const FieldDev& f, const TargetDev& t, int precision, const TrajArgs& a,
                         cudaStream_t s);
@@ -179,8 +180,23 @@ cudaError_t launch_redo(const FieldDev& f, const TargetDev& t, const TrajArgs& a
 // group lists of the four-warp redo: one per SM of the current device, at most kRedoLists
 constexpr int kRedoLists = 256;
 int redo_lists();
-// ints of device scratch the four-warp redo of a list of up to n births needs
-inline size_t redo_scratch_words(int64_t n) { return 3 * (size_t)kRedoLists + 2 * (size_t)((n + 31) / 32 + 1); }
+// trajectories per block of the four-lane kernel, and the longest list it takes
+constexpr int kQuadWidth = 8;
+int64_t quad_limit(int pot, int lists);
+// most groups of an escalation list of up to n births: 32 trajectories each, or 8 in a short list
+inline int64_t redo_groups(int64_t n, int64_t quad_limit) {
+    const int64_t q = n < quad_limit ? n : quad_limit;
+    const int64_t wide = (n + 31) / 32, quad = (q + kQuadWidth - 1) / kQuadWidth;
+    return (wide > quad ? wide : quad) + 1;
+}
+// ints of device scratch the redo of a list of up to n births needs (counters, list
+// lengths and starts, the groups list by list, each group's list)
+inline size_t redo_scratch_words(int64_t n, int64_t quad_limit) {
+    return 3 * (size_t)kRedoLists + 2 * (size_t)redo_groups(n, quad_limit);
+}
+cudaError_t launch_quad(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
+// the FP64 planar dipole of births [0, n) by the same kernels, without escalation list or scratch
+cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
 int64_t redo_blocks(int64_t n);
 // The high-precision pass over an escalation list: esc_precision 0 FP64 (the split
 // kernel where it applies: planar form, atomic bins), 1 double-float (planar form;

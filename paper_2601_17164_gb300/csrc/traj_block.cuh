@@ -113,6 +113,25 @@ __device__ __forceinline__ void potential_xz(R x, R z, const PotConst<R>& c, R& 
     }
 }
 
+// The Tong-Lin potential in FP64 in the pieces that the four-lane kernel (quad.cu) spreads
+// over warps, from r, 1/r and the three exponentials: Y and Y' (numerator of -V), g and h.
+// The fused operations are written out in the order that nvcc contracts potential_xz to in
+// the other FP64 kernels (found by comparing values over 1e6 positions): chaotic
+// trajectories follow the last bit of g, so the kernels agree only if every rounding does.
+__device__ __forceinline__ void tonglin_y(const PotConst<double>& c, double r, double e2, double e4, double e6,
+                                          double& Y, double& Y1) {
+    Y = fma(c.a5, e6, fma(c.a3 * r, e4, fma(c.a1, e2, c.Zc)));
+    Y1 = fma(-(c.a5 * c.a6), e6, fma(-c.a1 * c.a2t, e2, c.a3 * fma(-c.a4, r, 1.0) * e4));
+}
+__device__ __forceinline__ double tonglin_g(double ir, double Y, double Y1) { return fma(Y, ir, -Y1) * (ir * ir); }
+__device__ __forceinline__ double tonglin_h(const PotConst<double>& c, double r, double ir, double Y, double Y1,
+                                            double e2, double e4, double e6) {
+    const double w4 = c.a3 * fma(c.a4 * c.a4, r, -(2.0 * c.a4));
+    const double Y2 = fma(c.a5 * c.a6 * c.a6, e6, fma(c.a1 * c.a2t * c.a2t, e2, w4 * e4));
+    const double ir2 = ir * ir;
+    return (fma(3.0 * Y1, ir, -3.0 * Y * ir2) - Y2) * ir2 * ir;
+}
+
 // Action accumulator: plain in double; two-float reduced mod 2 pi in float.
 template <typename R>
 struct Action;
