@@ -75,87 +75,92 @@ __device__ __forceinline__ void philox4x64_10(uint64_t c[4], uint64_t k0, uint64
 
 // ---- analytic field on complex time ----------------------------------------
 // A(t) = sum_j a_j sin(w_j t + cep), E = -dA/dt, F = int_0^t A, G = int_0^t A^2.
-__device__ __forceinline__ cd field_A(const FieldDev& f, cd t) {
-    cd s = mk(0, 0);
-    for (int j = 0; j < f.n_modes; ++j) s = s + f.a[j] * c_sin(mk(f.w[j] * t.re + f.cep, f.w[j] * t.im));
-    return s;
-}
 __device__ __forceinline__ cd field_E(const FieldDev& f, cd t) {
     cd s = mk(0, 0);
     for (int j = 0; j < f.n_modes; ++j)
         s = s + (-f.a[j] * f.w[j]) * c_cos(mk(f.w[j] * t.re + f.cep, f.w[j] * t.im));
     return s;
 }
-// int_0^t cos(w s + th) ds for complex t
-__device__ __forceinline__ cd int_cos(double w, double th, cd t) {
-    if (fabs(w) < 1e-14) return cos(th) * t;
-    cd v = c_sin(mk(w * t.re + th, w * t.im));
-    return (1.0 / w) * (v - mk(sin(th), 0.0));
-}
-__device__ __forceinline__ cd field_F(const FieldDev& f, cd t) {
-    cd s = mk(0, 0);
-    for (int j = 0; j < f.n_modes; ++j) {
-        double w = f.w[j];
-        if (fabs(w) < 1e-14) {
-            s = s + (f.a[j] * sin(f.cep)) * t;
-        } else {
-            cd v = c_cos(mk(w * t.re + f.cep, w * t.im));
-            s = s + (f.a[j] / w) * (mk(cos(f.cep), 0.0) - v);
-        }
-    }
-    return s;
-}
-__device__ __forceinline__ cd field_G(const FieldDev& f, cd t) {
-    cd s = mk(0, 0);
-    for (int j = 0; j < f.n_modes; ++j)
-        for (int k = 0; k < f.n_modes; ++k) {
-            double c = 0.5 * f.a[j] * f.a[k];
-            s = s + c * (int_cos(f.w[j] - f.w[k], 0.0, t) - int_cos(f.w[j] + f.w[k], 2.0 * f.cep, t));
-        }
-    return s;
-}
-
-// The same four functions at one time from the sines and cosines of the mode phases
+// All four at one time from the sines and cosines of the mode phases
 // a_j = w_j t + cep, each computed once: A and E are sums over them, F a sum over
 // the cosines, and G's terms sin((w_j -+ w_k) t + ...) = sin(a_j -+ a_k) follow by
-// the angle-sum identities (no further transcendental calls).  At a real time the
-// hyperbolic factors (1 and 0) are left out.
+// the angle-sum identities (no further transcendental calls).
 struct FieldAt {
     cd A, E, F, G;
 };
-__device__ __forceinline__ FieldAt field_at(const FieldDev& f, cd t) {
+// The field's constants that every evaluation at a time would form the same way: sines and
+// cosines of cep and 2 cep, a_j/w_j and 1/(w_j -+ w_k) (0 where the divisor is below 1e-14).
+struct FieldConst {
+    double s_cep, c_cep, s_2cep, c_2cep;
+    double aw[3], im[3][3], ip[3][3];
+};
+// by the threads of a block (64 or more); the caller synchronises
+__device__ __forceinline__ void make_field_const(const FieldDev& f, FieldConst& c) {
+    const int v = threadIdx.x;
+    if (v == 0) sincos(f.cep, &c.s_cep, &c.c_cep);
+    if (v == 32) sincos(2.0 * f.cep, &c.s_2cep, &c.c_2cep);
+    if (v < 9) {
+        const int j = v / 3, k = v % 3;
+        const double wm = f.w[j] - f.w[k], wp = f.w[j] + f.w[k];
+        c.im[j][k] = fabs(wm) < 1e-14 ? 0.0 : 1.0 / wm;
+        c.ip[j][k] = fabs(wp) < 1e-14 ? 0.0 : 1.0 / wp;
+        if (k == 0) c.aw[j] = fabs(f.w[j]) < 1e-14 ? 0.0 : f.a[j] / f.w[j];
+    }
+}
+// sine and cosine of the mode phases w_j t + cep at a real time
+__device__ __forceinline__ void mode_phases(const FieldDev& f, double t, double sn[3], double cs[3]) {
+    const int nm = f.n_modes < 3 ? f.n_modes : 3;
+    for (int j = 0; j < nm; ++j) sincos(f.w[j] * t + f.cep, &sn[j], &cs[j]);
+}
+// at a complex t, whose real part has the mode phases sn, cs
+__device__ __forceinline__ FieldAt field_at(const FieldDev& f, cd t, const double sn[3], const double cs[3],
+                                            const FieldConst& fc) {
     cd s[3], c[3];
     const int nm = f.n_modes < 3 ? f.n_modes : 3;
-    for (int j = 0; j < nm; ++j) {
-        double sn, cs;
-        sincos(f.w[j] * t.re + f.cep, &sn, &cs);
-        if (t.im == 0.0) {
-            s[j] = mk(sn, 0.0);
-            c[j] = mk(cs, 0.0);
-        } else {
-            const double y = f.w[j] * t.im, ch = cosh(y), sh = sinh(y);
-            s[j] = mk(sn * ch, cs * sh);     // sin(x + i y)
-            c[j] = mk(cs * ch, -sn * sh);    // cos(x + i y)
-        }
-    }
-    double s_cep, c_cep, s_2cep, c_2cep;
-    sincos(f.cep, &s_cep, &c_cep);
-    sincos(2.0 * f.cep, &s_2cep, &c_2cep);
     FieldAt r{mk(0, 0), mk(0, 0), mk(0, 0), mk(0, 0)};
+    for (int j = 0; j < nm; ++j) {
+        const double y = f.w[j] * t.im, ch = cosh(y), sh = sinh(y);
+        s[j] = mk(sn[j] * ch, cs[j] * sh);     // sin(x + i y)
+        c[j] = mk(cs[j] * ch, -sn[j] * sh);    // cos(x + i y)
+    }
     for (int j = 0; j < nm; ++j) {
         const double a = f.a[j], w = f.w[j];
         r.A = r.A + a * s[j];
         r.E = r.E + (-a * w) * c[j];
-        if (fabs(w) < 1e-14) r.F = r.F + (a * s_cep) * t;
-        else r.F = r.F + (a / w) * (mk(c_cep, 0.0) - c[j]);
+        if (fc.aw[j] == 0.0) r.F = r.F + (a * fc.s_cep) * t;
+        else r.F = r.F + fc.aw[j] * (mk(fc.c_cep, 0.0) - c[j]);
     }
     for (int j = 0; j < nm; ++j)
         for (int k = 0; k < nm; ++k) {
             const double cf = 0.5 * f.a[j] * f.a[k];
-            const cd sc = s[j] * c[k], cs = c[j] * s[k];
-            const double wm = f.w[j] - f.w[k], wp = f.w[j] + f.w[k];
-            const cd im = fabs(wm) < 1e-14 ? t : (1.0 / wm) * (sc - cs);                           // int cos(wm s) ds
-            const cd ip = fabs(wp) < 1e-14 ? c_2cep * t : (1.0 / wp) * ((sc + cs) - mk(s_2cep, 0.0));  // int cos(wp s + 2 cep)
+            const cd sc = s[j] * c[k], cc = c[j] * s[k];
+            const cd im = fc.im[j][k] == 0.0 ? t : fc.im[j][k] * (sc - cc);                              // int cos(wm s) ds
+            const cd ip = fc.ip[j][k] == 0.0 ? fc.c_2cep * t : fc.ip[j][k] * ((sc + cc) - mk(fc.s_2cep, 0.0));  // int cos(wp s + 2 cep)
+            r.G = r.G + cf * (im - ip);
+        }
+    return r;
+}
+// the same at a real t: the real parts by the same operations (the imaginary ones are 0)
+struct FieldAt0 {
+    double A, E, F, G;
+};
+__device__ __forceinline__ FieldAt0 field_at_real(const FieldDev& f, double t, const double s[3], const double c[3],
+                                                  const FieldConst& fc) {
+    const int nm = f.n_modes < 3 ? f.n_modes : 3;
+    FieldAt0 r{0.0, 0.0, 0.0, 0.0};
+    for (int j = 0; j < nm; ++j) {
+        const double a = f.a[j], w = f.w[j];
+        r.A = r.A + a * s[j];
+        r.E = r.E + (-a * w) * c[j];
+        if (fc.aw[j] == 0.0) r.F = r.F + (a * fc.s_cep) * t;
+        else r.F = r.F + fc.aw[j] * (fc.c_cep - c[j]);
+    }
+    for (int j = 0; j < nm; ++j)
+        for (int k = 0; k < nm; ++k) {
+            const double cf = 0.5 * f.a[j] * f.a[k];
+            const double sc = __dmul_rn(s[j], c[k]), cc = __dmul_rn(c[j], s[k]);
+            const double im = fc.im[j][k] == 0.0 ? t : fc.im[j][k] * (sc - cc);
+            const double ip = fc.ip[j][k] == 0.0 ? fc.c_2cep * t : fc.ip[j][k] * ((sc + cc) - fc.s_2cep);
             r.G = r.G + cf * (im - ip);
         }
     return r;
