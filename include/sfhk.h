@@ -315,7 +315,8 @@ sfhk_status sfhk_resample_births(const sfhk_births* pool, int64_t m, int64_t n, 
  * block: threads per block (0 = library choice, 128; else 64 or 128).  An FP64
  * dipole call in the planar form without deterministic bins runs on the
  * warp-specialised kernels of the escalation pass when block = chunk_steps = 0
- * (no scratch), and with one thread per trajectory otherwise.
+ * (no scratch), FP64 endpoints on one of their own, and both with one thread
+ * per trajectory otherwise.
  * chunk_steps: steps per shared-memory field window (0 = library choice;
  * else a multiple of n_out, 64..8192).
  * ---------------------------------------------------------------------- */

@@ -744,12 +744,15 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
         a.esc_bin = esc_bin;
         a.esc_ratio = pp->esc_ratio;
     }
-    // FP64 planar dipole into atomic bins: the warp-specialised kernels; a caller's own
-    // launch shape (block, chunk_steps) asks for the one-thread-per-trajectory kernel
-    const bool warps64 = mode == 1 && pp->precision == 0 && a.planar && !det && pp->block == 0 && pp->chunk_steps == 0;
-    st = check_cuda(warps64 ? launch_fp64(field->f, target->t, a, s)
-                            : launch_traj(field->f, target->t, pp->precision, a, s),
-                    "trajectory launch");
+    // FP64 endpoints, and the FP64 planar dipole into atomic bins: the warp-specialised
+    // kernels; a caller's own launch shape (block, chunk_steps) asks for the
+    // one-thread-per-trajectory kernel
+    const bool warps64 = pp->precision == 0 && pp->block == 0 && pp->chunk_steps == 0;
+    cudaError_t launched;
+    if (warps64 && mode == 0) launched = launch_endpoints(field->f, target->t, a, s);
+    else if (warps64 && a.planar && !det) launched = launch_fp64(field->f, target->t, a, s);
+    else launched = launch_traj(field->f, target->t, pp->precision, a, s);
+    st = check_cuda(launched, "trajectory launch");
     if (st) return st;
     if (det) {
         st = check_cuda(launch_reduce_partials(part, n_blocks, field->f.n_bins, d_len, d_vel, s), "reduce launch");

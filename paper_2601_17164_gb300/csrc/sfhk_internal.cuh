@@ -172,6 +172,8 @@ struct TrajArgs {
 };
 cudaError_t launch_traj(const FieldDev& f, const TargetDev& t, int precision, const TrajArgs& a,
                         cudaStream_t s);
+// FP64 endpoints of the full state, eight warps per 32 trajectories (endpoints.cu)
+cudaError_t launch_endpoints(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
 // 32-bit words of saved state per birth in a segmented float pass (planar or 3D form)
 int state_words(int planar);
 // FP64 redo of an escalation list (planar form, atomic bins) with the work of each
