@@ -13,8 +13,11 @@
 // in float with an error bound, 16 points at a time, skipping a run that a slope bound
 // shows to be free of roots; a point whose sign the bound leaves open is evaluated in
 // FP64.  Per-target constants and the sines and cosines at a birth's time are formed
-// once.  Measured at 1e6 births (H, 800 nm, 8 cycles): 30.0 ms with the scan in FP64,
-// 9.2 ms now.
+// once.  The Newton iteration takes 4 steps for half of the births and up to 48 where it
+// ends in bisection, so the lanes of a block take their problems from a queue over its
+// births (4 per thread in a large call) instead of waiting for the slowest of 32.
+// Measured at 1e6 births (H, 800 nm, 8 cycles): 30.0 ms with the scan in FP64, 9.2 ms
+// with the scan in float, 6.0 ms with the queue.
 #include "sfhk_device.cuh"
 
 namespace sfhk {
@@ -54,9 +57,15 @@ __device__ cd tunnel_element(const TargetDev& t, const BirthConst& bc, cd kx, cd
     return pw * s;
 }
 
-// Smallest root of f(tau) = sum_j c_j sinh(w_j tau) - target on (0, tau_max].
-// cs[j]: cos(w_j t0 + cep).
-__device__ bool solve_tt(const FieldDev& f, const double* cs, double target, double* tt) {
+// The saddle's equation f(tau) = sum_j c_j sinh(w_j tau) - target, c_j = a_j cos(w_j t0 +
+// cep) (cs[j]: the cosines): the grid cell [(hit - 1) h, hit h] of its smallest root on
+// (0, 25/w_max], h = 0.02/w_max; 0 when there is none.
+__device__ __forceinline__ double scan_step(const FieldDev& f) {
+    double wmax = 0.0;
+    for (int j = 0; j < f.n_modes; ++j) wmax = fmax(wmax, fabs(f.w[j]));
+    return wmax == 0.0 ? 0.0 : 0.02 / wmax;
+}
+__device__ int scan_root(const FieldDev& f, const double* cs, double target) {
     double c[3], w[3];
     double wmax = 0.0;
     for (int j = 0; j < f.n_modes; ++j) {
@@ -64,7 +73,7 @@ __device__ bool solve_tt(const FieldDev& f, const double* cs, double target, dou
         w[j] = f.w[j];
         wmax = fmax(wmax, fabs(w[j]));
     }
-    if (wmax == 0.0) return false;
+    if (wmax == 0.0) return 0;
     const double h = 0.02 / wmax, tmax = 25.0 / wmax;
     const int nscan = (int)(tmax / h);
     // The first grid point it h at which f has left the sign of f(0) = -target.  Float
@@ -123,34 +132,42 @@ __device__ bool solve_tt(const FieldDev& f, const double* cs, double target, dou
             }
         }
     }
-    if (!hit) return false;
-    const double tau = hit * h;
-    double lo = tau - h, hi = tau;
-    // safeguarded Newton inside the bracket (bisection when a step leaves it)
-    double x = 0.5 * (lo + hi);
-    for (int it = 0; it < 100; ++it) {
+    return hit;
+}
+
+// The root in that cell: safeguarded Newton inside the bracket (bisection when a step
+// leaves it), one step at a time.
+struct Newton {
+    double c[3], target, lo, hi, x;
+    int it;
+    __device__ __forceinline__ void start(const FieldDev& f, const double cs[3], double goal, int hit, double h) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) c[j] = j < f.n_modes ? f.a[j] * cs[j] : 0.0;
+        target = goal;
+        const double tau = hit * h;
+        lo = tau - h;
+        hi = tau;
+        x = 0.5 * (lo + hi);
+        it = 0;
+    }
+    // true when done: the root is x
+    __device__ __forceinline__ bool step(const FieldDev& f) {
         double v = -target, d = 0.0;
-        for (int j = 0; j < f.n_modes; ++j) {
-            const double e = exp(w[j] * x), ie = 1.0 / e;
-            v += c[j] * 0.5 * (e - ie);          // sinh
-            d += c[j] * w[j] * 0.5 * (e + ie);   // derivative: w cosh
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (j >= f.n_modes) break;
+            const double e = exp(f.w[j] * x), ie = 1.0 / e;
+            v += c[j] * 0.5 * (e - ie);            // sinh
+            d += c[j] * f.w[j] * 0.5 * (e + ie);   // derivative: w cosh
         }
-        if ((v > 0) == up0) lo = x; else hi = x;   // f has the sign of f(0) at lo
+        if ((v > 0) == (-target > 0.0)) lo = x; else hi = x;   // f has the sign of f(0) at lo
         double xn = (d != 0.0) ? x - v / d : 0.5 * (lo + hi);
         if (!(xn > lo && xn < hi)) xn = 0.5 * (lo + hi);
         const bool done = fabs(xn - x) <= 1e-15 * fabs(xn) || hi - lo <= 1e-15 * hi;
         x = xn;
-        if (done) break;
+        return done || ++it == 100;
     }
-    *tt = x;
-    return true;
-}
-
-// The saddle of a birth (t0, kx, ky) and its amplitude without the Monte Carlo
-// measure: kind 0 standard SPA, 1 modified SPA, 2 ADK (modulus sqrt(adk_n2 rho),
-// phase Re S, exit q0 = -Ip/E(t0), kz = 0).  Returns false where no saddle exists.
-__device__ bool birth_amp(const FieldDev& f, const TargetDev& t, const BirthConst& bc, double t0, double kx, double ky,
-                          int kind, double adk_n2, double* kz_out, double* qz_out, cd* amp_out);
+};
 
 // ADK rate per unit time (Z_c = 1, m = 0, l = gto_l; the tail constant C_l^2 left out):
 //   w(F) = (2l+1)/2 kappa^{1-2/kappa} (2 kappa^3/F)^{2/kappa-1} exp(-2 kappa^3/(3F)),
@@ -167,21 +184,28 @@ __device__ double adk_density(const TargetDev& t, double F, double kperp2) {
     return adk_rate(t, F) * kappa / (kPi * F) * exp(-kappa * kperp2 / F);
 }
 
-__device__ bool birth_amp(const FieldDev& f, const TargetDev& t, const BirthConst& bc, double t0, double kx, double ky,
-                          int kind, double adk_n2, double* kz_out, double* qz_out, cd* amp_out) {
-    *kz_out = 0.0;
-    *qz_out = 0.0;
-    *amp_out = mk(0, 0);
-    double sn0[3], cs0[3];
-    mode_phases(f, t0, sn0, cs0);
-    const FieldAt0 at0 = field_at_real(f, t0, sn0, cs0, bc.fc);
-    const double Et0 = at0.E;
-    if (Et0 == 0.0) return false;
+// A birth at (t0, kx, ky) with the mode phases sn0, cs0: its side of the saddle's equation
+// (0 where the field vanishes and there is no saddle).
+__device__ __forceinline__ double saddle_target(const FieldDev& f, const TargetDev& t, const double cs0[3], double kx,
+                                                double ky) {
+    double Et0 = 0.0;
+    for (int j = 0; j < f.n_modes; ++j) Et0 = Et0 + (-f.a[j] * f.w[j]) * cs0[j];
+    if (Et0 == 0.0) return 0.0;
     const double kp2 = kx * kx + ky * ky;
     const double kappa = sqrt(2.0 * t.ip + kp2);
     const double s = Et0 > 0 ? -1.0 : 1.0;
-    double tt;
-    if (!solve_tt(f, cs0, s * kappa, &tt)) return false;
+    return s * kappa;
+}
+
+// The saddle of a birth at t0 + i tt and its amplitude without the Monte Carlo measure:
+// kind 0 standard SPA, 1 modified SPA, 2 ADK (modulus sqrt(adk_n2 rho), phase Re S, exit
+// q0 = -Ip/E(t0), kz = 0).
+__device__ void birth_amp(const FieldDev& f, const TargetDev& t, const BirthConst& bc, double t0, double tt,
+                          const double sn0[3], const double cs0[3], double kx, double ky, int kind, double adk_n2,
+                          double* kz_out, double* qz_out, cd* amp_out) {
+    const FieldAt0 at0 = field_at_real(f, t0, sn0, cs0, bc.fc);
+    const double Et0 = at0.E;
+    const double kp2 = kx * kx + ky * ky;
     const cd ts = mk(t0, tt);
     const FieldAt ats = field_at(f, ts, sn0, cs0, bc.fc);
     const double A0 = at0.A;
@@ -217,7 +241,6 @@ __device__ bool birth_amp(const FieldDev& f, const TargetDev& t, const BirthCons
     *kz_out = kz;
     *qz_out = qz;
     *amp_out = amp;
-    return true;
 }
 
 // ADK renormalisation N^2 (Sec. III.C), evaluated by every block of 128 threads
@@ -240,9 +263,18 @@ __device__ double adk_norm2_block(const FieldDev& f, const TargetDev& t, BirthCo
             const int i = 2 * m + 1 + q;
             const double k = (double)i * h;
             const double c = (i == 128) ? 1.0 : ((i & 1) ? 4.0 : 2.0);
-            double kz, qz;
+            double sn[3], cs[3], kz, qz;
+            mode_phases(f, tj, sn, cs);
+            const double goal = saddle_target(f, t, cs, k, 0.0);
+            const int hit = goal != 0.0 ? scan_root(f, cs, goal) : 0;
+            if (hit == 0) continue;
+            Newton nw;
+            nw.start(f, cs, goal, hit, scan_step(f));
+            while (!nw.step(f)) {
+            }
             cd a;
-            if (birth_amp(f, t, bc, tj, k, 0.0, 0, 0.0, &kz, &qz, &a)) part += c * k * (a.re * a.re + a.im * a.im);
+            birth_amp(f, t, bc, tj, nw.x, sn, cs, k, 0.0, 0, 0.0, &kz, &qz, &a);
+            part += c * k * (a.re * a.re + a.im * a.im);
         }
     }
     s_part[tid] = part;
@@ -261,12 +293,11 @@ __device__ double adk_norm2_block(const FieldDev& f, const TargetDev& t, BirthCo
     return (den > 0.0 && isfinite(n2)) ? n2 : 0.0;
 }
 
-// Birth o of the produced range (output index).
-__device__ void one_birth(const FieldDev& f, const TargetDev& t, const BirthArgs& a, const BirthConst& bc,
-                          double adk_n2, int64_t o) {
+// The draws of birth o of the produced range (output index): its step and transverse
+// momentum, and its Monte Carlo measure.
+__device__ void draw_birth(const FieldDev& f, const BirthArgs& a, int64_t o, int64_t& nb, double& kx, double& ky,
+                           double& w) {
     const int64_t i = a.first + o;                                       // birth index
-    int64_t nb;
-    double kx, ky, w;
     const int64_t M = f.n_steps - 1;
     if (a.mode == 0) {
         int64_t it = i / a.n_k, ik = i % a.n_k;
@@ -294,39 +325,112 @@ __device__ void one_birth(const FieldDev& f, const TargetDev& t, const BirthArgs
         // w = 1/(n pdf),  pdf = e^{-k^2/2s^2}/(2 pi s^2) * 1/(M dt)
         w = 2.0 * kPi * s2 * exp((kx * kx + ky * ky) / (2.0 * s2)) * ((double)M * f.dt) / (double)a.n;
     }
-    const double t0 = f.t_start + (double)nb * f.dt;
-    double kz = 0.0, qz = 0.0;
-    cd amp = mk(0, 0);
-    birth_amp(f, t, bc, t0, kx, ky, t.amp, adk_n2, &kz, &qz, &amp);
-    a.n0[o] = (int32_t)nb;
-    a.t0[o] = t0;
-    a.px[o] = kx;
-    a.py[o] = ky;
-    a.pz[o] = kz;
-    a.qz[o] = qz;
-    a.amp_re[o] = w * amp.re;
-    a.amp_im[o] = w * amp.im;
 }
 
-__global__ void __launch_bounds__(128) births_kernel(FieldDev f, TargetDev t, BirthArgs a) {
+constexpr int kThreads = 128;   // the ADK renormalisation spreads its 2 x 64 Simpson pairs over 128 threads
+
+// R births per thread and tile, between the draws and the amplitudes in shared memory
+template <int R>
+struct BirthTile {
+    double sn[3][R * kThreads], cs[3][R * kThreads];
+    double root[R * kThreads];   // the equation's target, then its root
+    double w[R * kThreads];
+    int hit[R * kThreads];
+    int next;
+};
+
+template <int R>
+__global__ void __launch_bounds__(kThreads, 2) births_kernel(FieldDev f, TargetDev t, BirthArgs a) {
     __shared__ BirthConst bc;
+    __shared__ BirthTile<R> tl;
     make_const(f, t, bc);
     const double adk_n2 = t.amp == 2 ? adk_norm2_block(f, t, bc) : 0.0;   // every thread takes part
-    for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < a.count;
-         o += (int64_t)gridDim.x * blockDim.x)
-        one_birth(f, t, a, bc, adk_n2, o);
+    const double h = scan_step(f);
+    constexpr int kTile = R * kThreads;
+    for (int64_t o0 = (int64_t)blockIdx.x * kTile; o0 < a.count; o0 += (int64_t)gridDim.x * kTile) {
+        const int nt = (int)(a.count - o0 < kTile ? a.count - o0 : kTile);
+        // draws and brackets
+        for (int u = threadIdx.x; u < nt; u += kThreads) {
+            const int64_t o = o0 + u;
+            int64_t nb;
+            double kx, ky, w, sn[3], cs[3];
+            draw_birth(f, a, o, nb, kx, ky, w);
+            const double t0 = f.t_start + (double)nb * f.dt;
+            mode_phases(f, t0, sn, cs);
+            const double goal = saddle_target(f, t, cs, kx, ky);
+            tl.hit[u] = goal != 0.0 ? scan_root(f, cs, goal) : 0;
+            tl.root[u] = goal;
+            tl.w[u] = w;
+            for (int j = 0; j < f.n_modes; ++j) {
+                tl.sn[j][u] = sn[j];
+                tl.cs[j][u] = cs[j];
+            }
+            a.n0[o] = (int32_t)nb;
+            a.t0[o] = t0;
+            a.px[o] = kx;
+            a.py[o] = ky;
+        }
+        if (threadIdx.x == 0) tl.next = 0;
+        __syncthreads();
+        // roots: every lane iterates on one birth and then takes the next
+        {
+            Newton nw;
+            int u = -1;
+            for (;;) {
+                while (u < 0) {
+                    u = atomicAdd(&tl.next, 1);
+                    if (u >= nt) break;
+                    if (tl.hit[u] == 0) {
+                        u = -1;
+                        continue;
+                    }
+                    const double cs[3] = {tl.cs[0][u], tl.cs[1][u], tl.cs[2][u]};
+                    nw.start(f, cs, tl.root[u], tl.hit[u], h);
+                }
+                if (u >= nt) break;
+                if (nw.step(f)) {
+                    tl.root[u] = nw.x;
+                    u = -1;
+                }
+            }
+        }
+        __syncthreads();
+        // amplitudes
+        for (int u = threadIdx.x; u < nt; u += kThreads) {
+            const int64_t o = o0 + u;
+            double kz = 0.0, qz = 0.0;
+            cd amp = mk(0, 0);
+            if (tl.hit[u]) {
+                double sn[3], cs[3];
+                for (int j = 0; j < f.n_modes; ++j) {
+                    sn[j] = tl.sn[j][u];
+                    cs[j] = tl.cs[j][u];
+                }
+                birth_amp(f, t, bc, a.t0[o], tl.root[u], sn, cs, a.px[o], a.py[o], t.amp, adk_n2, &kz, &qz, &amp);
+            }
+            const double w = tl.w[u];
+            a.pz[o] = kz;
+            a.qz[o] = qz;
+            a.amp_re[o] = w * amp.re;
+            a.amp_im[o] = w * amp.im;
+        }
+        __syncthreads();   // the tile is free
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_births(const FieldDev& f, const TargetDev& t, const BirthArgs& a, cudaStream_t s) {
     if (a.count == 0) return cudaSuccess;
-    const int block = 128;   // the ADK renormalisation spreads its 2 x 64 Simpson pairs over 128 threads
-    int64_t grid = (a.count + block - 1) / block;
+    // four births per thread where that still fills the chip (2 blocks on each of 152 SMs);
     // ADK: every block evaluates the renormalisation (two births a thread), so no more
-    // blocks than are resident at once (2 on each of 152 SMs), each on several tiles
+    // blocks than are resident at once, each on several tiles
+    const bool large = a.count >= (int64_t)4 * kThreads * 304;
+    const int64_t tile = large ? 4 * kThreads : kThreads;
+    int64_t grid = (a.count + tile - 1) / tile;
     if (t.amp == 2 && grid > 304) grid = 304;
-    births_kernel<<<(unsigned)grid, block, 0, s>>>(f, t, a);
+    if (large) births_kernel<4><<<(unsigned)grid, kThreads, 0, s>>>(f, t, a);
+    else births_kernel<1><<<(unsigned)grid, kThreads, 0, s>>>(f, t, a);
     return cudaGetLastError();
 }
 
