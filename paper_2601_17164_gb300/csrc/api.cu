@@ -669,6 +669,7 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
                 e.k_from = kfrom + c0;
                 e.count = count + c;
                 e.redo_ctr = rctr + (size_t)c * rw;
+                e.redo_shift = c * (a.redo_lists / kSide);
                 st = check_cuda(launch_escalation(field->f, target->t, epr, e, side), "escalation launch");
                 if (st) return st;
                 st = check_cuda(cudaEventRecord(sp->done[c], side), "event record");
@@ -721,6 +722,7 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
             e.k_from = kf_g;
             e.count = count + g;
             e.redo_ctr = rctr + (size_t)g * rw;
+            e.redo_shift = g * (a.redo_lists / kSide);
             st = check_cuda(launch_escalation(field->f, target->t, epr, e, side), "escalation launch");
             if (st) return st;
             st = check_cuda(cudaEventRecord(sp->done[g], side), "event record");

@@ -340,6 +340,7 @@ sfhk_status sfhk_batch_run(sfhk_batch* b, void* stream) {
         e.count = b->d_count + c;
         e.redo_lists = redo_lists();
         e.quad_limit = quad_limit(cfg.t.pot, e.redo_lists);
+        e.redo_shift = (c % 8) * (e.redo_lists / 8);   // the side streams' redos run side by side
         e.redo_ctr = b->d_rctr + (size_t)(c % 8) * b->rctr_words;
         st = check_cuda(launch_escalation(cfg.f, cfg.t, b->esc_precision, e, side), "escalation launch");
         if (st) return st;

@@ -9,18 +9,24 @@
 // dynamics warp while most SMs idle.  Here a block of four warps holds 8
 // trajectories and every trajectory has four lanes, which split the work inside a
 // step so that one instruction does four parts of it:
-//   dynamics  lanes = {x', z} x {q, p}: one FMA forms the next stage's positions and
-//             momenta, one chain the RK4 combination of all four; the Tong-Lin
-//             potential's three exponentials are one (lanes 0..2);
+//   dynamics  lanes = {x', z} x {stages 1 and 3, stages 2 and 4}: the force does not
+//             depend on the momentum, so two stages run side by side; the RK4
+//             combination of q in the one pair, of p in the other;
 //   matrix    lane s forms stage s's Hessian and action integrand, then lane (i, j)
 //             the entries (i, j) of A, B, C and D;
 //   columns   lane c advances column c, lane k one entry of the out-of-plane block;
-//   bins      lane j forms column j of Z, even lanes the real and odd lanes the
-//             imaginary part of det Z; the GTO terms of an FP64 bin in four parts.
-// FP64 instructions per step: dynamics 84 -> 48 (soft-core), 380 -> 160
-// (Tong-Lin), the whole step 323 -> 135 per 8 trajectories: one block per SM steps
-// 2.1 times as fast as 32 trajectories a block, with 1.7 times the FP64 work per
-// trajectory, so the host and the plan choose by list length (quad_limit).
+//   bins      labels, removal and the recombination terms, those of an FP64 bin in four
+//             parts, with the two phases of the bin in one sincos;
+// det Z (lane j forms column j of Z, even lanes the real and odd lanes the imaginary part)
+// goes to the bins warp when the recombination terms are formed in float, to the columns
+// warp when FP64 terms load the bins warp.
+// FP64 instructions per step: dynamics 84 -> 29 (soft-core), 380 -> 111 (Tong-Lin), the
+// four warps 29, 28, 33, 29 (float bins, soft-core): a block alone on its SM steps in
+// 2,900 cycles instead of the 7,600 of 32 trajectories a block (Tong-Lin: 8,500 instead
+// of 24,200), with 1.5 times the FP64 work per trajectory, so the host and the plan
+// choose by list length (quad_limit).  Measured: mixed H 8 cycles, 4096 births (110
+// redone) 334 -> 170 ms; mixed Ar 6 cycles, 5e4 births 1730 -> 660 ms; FP64 H 2 cycles,
+// 1024 births 140.6 -> 21.3 ms.
 //
 // Every value is formed by the same operations in the same order as in TrajP
 // (traj_block.cuh): trajectories, columns, determinants, branches and removals are
@@ -36,20 +42,29 @@ namespace {
 
 constexpr int kT = kQuadWidth;   // trajectories per block
 constexpr int kThreads = 128;
-// dynamics -> matrix, per stage: q (2), g, aux, p (2), then Tong-Lin: Y, Y1, e2, e4, e6;
+// dynamics -> matrix, per stage: q (2), g, 1/r, p (2), then soft-core: 1/r^2 (r with the
+// core's radius), Tong-Lin: Y, Y1, e2, e4, e6;
 // the stage stride puts lanes of neighbouring stages on different banks
 constexpr int kFields = 12;
 constexpr int kStage = kFields * kT + kT;
-// matrix -> columns: A, B, C, D (4 entries each), the out-of-plane rows (a, b), (c, d), state, S
-constexpr int kM = 16, kState = 20, kAct = 24, kN12 = 25;
-// columns -> bins: columns (4 x 4), out-of-plane (4), state, S
-constexpr int kN23 = 25;
+// matrix -> columns: A, B, C, D (4 entries each), the out-of-plane rows (a, b), (c, d) or
+// (float bins) g of the stages, state, the action's integrand at the four stages
+constexpr int kM = 16, kState = 20, kAct = 24, kN12 = 28;
+// columns -> bins: state at grid point n, then (float bins) the action there, the columns
+// after the step (4 x 4) and the out-of-plane block (4), or the action's four integrands,
+// 8 det Z (2) and its branch at grid point n
+constexpr int kDetF = 5, kDetD = 8, kN23 = 25;
+
+// barrier bases of the three hand-offs; the last one has three slots, which the bins warp's
+// longer grid points (those with a bin) need
+constexpr int kHand0 = 1, kHand1 = 5, kHand2 = 9;
 
 struct QShared {
     double s01[2][4 * kStage];
     double s12[2][kN12 * kT];
-    double s23[2][kN23 * kT];
+    double s23[3][kN23 * kT];
     double hess[4 * 3 * kT];   // stage Hessians (a, b, c), matrix warp only
+    double phase[16][2];       // cos and -sin of Ip t at bin k in row k & 15 (float bins)
     int alive[kT];             // written by the bins warp, read late by the warps ahead
 };
 
@@ -75,86 +90,123 @@ __device__ __forceinline__ PotConst<double> pot_const(const TargetDev& tg) {
     return pc;
 }
 
-// dynamics: the state at grid point n and the stages of the step n -> n + 1.  Lane
-// (component c = l & 1, kind l >> 1): kind 0 carries q_c, kind 1 p_c.
-template <int POT>
+// Ip t mod 2 pi at grid point n
+__device__ __forceinline__ double bin_phase(const FieldDev& f, const TargetDev& tg, int64_t n) {
+    return fmod_2pi(tg.ip * (f.t_start + (double)n * f.dt));
+}
+
+// dynamics: the state at grid point n and the stages of the step n -> n + 1.  The force
+// does not depend on the momentum, so the RK4 positions are
+//   Q1, Q2 = Q1 + h/2 P1, Q3 = Q1 + h/2 P2, Q4 = Q1 + h P3,
+//   P2 = P1 + h/2 F(Q1), P3 = P1 + h/2 F(Q2), P4 = P1 + h F(Q3):
+// the forces of stages 1 and 2 are formed side by side, then those of 3 and 4.  Lane
+// (component c = l & 1, pair g = l >> 1) takes stages 1 and 3 (g = 0) or 2 and 4.
+template <int POT, bool FB>
 __device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const TrajArgs& a, const QCommon& cm,
                               QShared& sm) {
     const PotConst<double> pc = pot_const<POT>(tg);
-    const int t = cm.t, c = cm.l & 1;
-    const bool isp = cm.l >= 2;
-    double b;   // this lane's part of the state
+    const int t = cm.t, c = cm.l & 1, pair = cm.l >> 1;
+    double q1, p1;   // this lane's component of the state
     {
         TrajP<double, POT> T;
         T.init(0.0, 0.0, cm.have ? a.qz[cm.i] : 0.0, cm.have ? a.px[cm.i] : 0.0, cm.have ? a.py[cm.i] : 0.0,
                cm.have ? a.pz[cm.i] : 0.0);
-        b = isp ? (c ? T.p[2] : T.p[0]) : (c ? T.q[2] : T.q[0]);
+        q1 = c ? T.q[2] : T.q[0];
+        p1 = c ? T.p[2] : T.p[0];
     }
     const StepK<double> hk = f.k64;
     const double* E = f.E64;
     auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(E + j) : 0.0; };
     double e0 = e_at(2 * cm.n_first), e1 = e_at(2 * cm.n_first + 1), e2 = e_at(2 * cm.n_first + 2);
     const volatile int* alive = sm.alive;
-    // Tong-Lin: this lane's exponent
-    const double ea = POT == POT_TONGLIN ? -(cm.l == 0 ? pc.a2t : (cm.l == 1 ? pc.a4 : pc.a6)) : 0.0;
-    Producer out(0);
+    // Tong-Lin: this lane's first exponent, and its constants of Y (c = 0) or Y' (c = 1)
+    const double ea = c ? -pc.a4 : -pc.a2t, t_r = c ? -pc.a4 : 1.0, t_1 = c ? 1.0 : 0.0, t_0 = c ? 0.0 : pc.Zc,
+                 t_2 = c ? -pc.a1 * pc.a2t : pc.a1, t_6 = c ? -(pc.a5 * pc.a6) : pc.a5;
+    Producer<2> out(kHand0);
+    // the force at a stage from this lane's component q of its position; the stage's
+    // Hessian data into the slot at os
+    auto force = [&](double q, double ek, double* os, double& g) {
+        const double qo = xor_lane(q, kT);
+        const double x = c ? qo : q, z = c ? q : qo;
+        double aux = 0.0;
+        if constexpr (POT == POT_SOFTCORE) {
+            const double r2 = fma(x, x, fma(z, z, pc.a2));
+            const double s = rsq(r2);
+            const double s2 = s * s;
+            g = s2 * s;
+            aux = s;
+            if (c == 0) os[6 * kT] = s2;
+        } else if constexpr (POT == POT_TONGLIN) {
+            const double r2 = fma(x, x, z * z);
+            const double ir = rsq(r2);
+            const double r = r2 * ir;
+            const double ex_l = ex(ea * r), x6 = ex(-pc.a6 * r);
+            const double ex_o = xor_lane(ex_l, kT);
+            const double x2 = c ? ex_o : ex_l, x4 = c ? ex_l : ex_o;
+            // Y in even and Y' in odd lanes, 5 instructions instead of 9
+            const double t3 = pc.a3 * fma(t_r, r, t_1);
+            const double v = fma(c ? t3 : t_2, c ? x4 : x2, t_0);
+            const double yl = fma(t_6, x6, fma(c ? t_2 : t3, c ? x2 : x4, v));
+            const double yo = xor_lane(yl, kT);
+            g = tonglin_g(ir, c ? yo : yl, c ? yl : yo);
+            aux = ir;
+            os[(6 + c) * kT] = yl;
+            os[(8 + c) * kT] = ex_l;
+            if (c == 0) os[10 * kT] = x6;
+        } else if constexpr (POT == POT_HARMONIC) {
+            g = pc.a2;
+        } else {
+            g = 0.0;
+        }
+        os[c * kT] = q;                       // q_x', q_z
+        os[(2 + c) * kT] = c ? aux : g;       // g, aux
+        return -fma(g, q, c ? ek : 0.0);      // -g x' and -(g z + E)
+    };
+    int rem = (int)(cm.n_first % cm.n_out);
+    int64_t k_bin = (cm.n_first + cm.n_out - 1) / cm.n_out;
     for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
         const int d = out.acquire();
+        // float bins: e^{-i Ip t} of the bin at this grid point (this warp has the FP64
+        // instructions to spare; the hand-offs keep the bins warp less than 16 grid points
+        // behind, so a row is read before its next use even with a bin at every point)
+        if (FB && rem == 0) {
+            if (threadIdx.x % 32 == 0) {
+                double sn, cs;
+                sincos(bin_phase(f, tg, n), &sn, &cs);
+                sm.phase[k_bin & 15][0] = cs;
+                sm.phase[k_bin & 15][1] = -sn;
+            }
+            ++k_bin;
+        }
+        rem = (rem + 1 == cm.n_out) ? 0 : rem + 1;
         double* const o = sm.s01[d] + t;
         const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
         const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
-        double y = b, u[4], m3 = 1.0, v3 = 0.0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            // positions of the stage in every lane; the stage momentum in the q lanes
-            const double x = from_lane(y, t), z = from_lane(y, t + kT);
-            const double pk = from_lane(y, t + (2 + c) * kT);
-            double g, aux = 0.0, Y = 0.0, Y1 = 0.0, ex_l = 0.0;
-            if constexpr (POT == POT_SOFTCORE) {
-                const double r2 = fma(x, x, fma(z, z, pc.a2));
-                const double s = rsq(r2);
-                const double s2 = s * s;
-                g = s2 * s;
-                aux = s;
-            } else if constexpr (POT == POT_TONGLIN) {
-                const double r2 = fma(x, x, z * z);
-                const double ir = rsq(r2);
-                const double r = r2 * ir;
-                ex_l = ex(ea * r);
-                const double x2 = from_lane(ex_l, t), x4 = from_lane(ex_l, t + kT), x6 = from_lane(ex_l, t + 2 * kT);
-                tonglin_y(pc, r, x2, x4, x6, Y, Y1);
-                g = tonglin_g(ir, Y, Y1);
-                aux = ir;
-            } else if constexpr (POT == POT_HARMONIC) {
-                g = pc.a2;
-            } else {
-                g = 0.0;
-            }
-            // -g x' and -(g z + E)
-            const double ek = k == 0 ? e0 : (k == 3 ? e2 : e1);
-            const double kp = -fma(g, c ? z : x, c ? ek : 0.0);
-            u[k] = isp ? kp : pk;
-            double* const os = o + k * kStage;
-            os[cm.l * kT] = isp ? (c ? aux : g) : y;                                    // q_x', q_z, g, aux
-            if constexpr (POT == POT_TONGLIN) {
-                os[(isp ? 4 + c : 6 + c) * kT] = isp ? y : (c ? Y1 : Y);                // p_x', p_z, Y, Y1
-                if (cm.l < 3) os[(8 + cm.l) * kT] = ex_l;
-            } else {
-                if (isp) os[(4 + c) * kT] = y;
-            }
-            if (k < 3) y = fma(k < 2 ? hk.hh : hk.h, u[k], b);
-            else {
-                // the last term of the p_x' combination is -g x' unrounded (so nvcc contracts
-                // it in the other FP64 kernels: found by comparing chaotic trajectories)
-                const bool px = isp && c == 0;
-                m3 = px ? -g : 1.0;
-                v3 = px ? x : u[3];
-            }
-        }
-        // the RK4 combination of this lane's component
-        const double nb = fma(hk.h6, fma(m3, v3, fma(2.0, u[1] + u[2], u[0])), b);
-        if (step) b = nb;
+        double g;
+        const double qa = pair ? fma(hk.hh, p1, q1) : q1;                       // Q1, Q2
+        const double ka = force(qa, pair ? e1 : e0, o + pair * kStage, g);      // F1, F2
+        const double pn = fma(hk.hh, ka, p1);                                   // P2, P3
+        const double qb = fma(pair ? hk.h : hk.hh, pn, q1);                     // Q3, Q4
+        const double kb = force(qb, pair ? e2 : e1, o + (2 + pair) * kStage, g);   // F3, F4
+        const double p4 = fma(hk.h, kb, p1);                                    // (P4 in the first pair)
+        // stage momenta: P2 and P3, P1 and P4
+        o[(1 + pair) * kStage + (4 + c) * kT] = pn;
+        const double p4_o = xor_lane(p4, 2 * kT);
+        o[(pair ? 3 * kStage : 0) + (4 + c) * kT] = pair ? p4_o : p1;
         out.publish(d);
+        // the RK4 combination, q_c in the first pair and p_c in the second; the last term of
+        // p_x' is -g x' unrounded (so nvcc contracts it in the other FP64 kernels: found by
+        // comparing chaotic trajectories)
+        const double pn_o = xor_lane(pn, 2 * kT), ka_o = xor_lane(ka, 2 * kT), kb_o = xor_lane(kb, 2 * kT);
+        const double s3 = fma(2.0, (pair ? ka : pn) + (pair ? kb_o : pn_o), pair ? ka_o : p1);
+        const bool px = pair && c == 0;
+        const double s = fma(px ? -g : 1.0, px ? qb : (pair ? kb : p4), s3);
+        const double nb = fma(hk.h6, s, pair ? p1 : q1);
+        const double no = xor_lane(nb, 2 * kT);
+        if (step) {
+            q1 = pair ? no : nb;
+            p1 = pair ? nb : no;
+        }
         e0 = f0;
         e1 = f1;
         e2 = f2;
@@ -162,8 +214,51 @@ __device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const Traj
     out.drain();
 }
 
-// matrix: the step matrix of grid point n and the action
-template <int POT>
+// the out-of-plane rows: (a, b) in even lanes, (c, d) in odd lanes (TrajP::step_matrix)
+__device__ __forceinline__ double2 out_of_plane(const StepK<double>& k, double g0, double g1, double g2, double g3,
+                                                bool odd) {
+    const double g23 = g1 + g2;
+    const double ad = fma(k.c4, (odd ? g3 : g2) * (odd ? g1 : g0), -k.c2 * (g23 + (odd ? g3 : g0)));
+    const double w = fma(g2, g0, g3 * g1), v = -k.h6 * (fma(2.0, g23, g0) + g3);
+    const double bc = fma(odd ? k.c3 : -k.c3, odd ? w : g23, odd ? v : k.h);
+    return odd ? make_double2(bc, ad) : make_double2(ad, bc);
+}
+
+// 8 det Z (of 2 Z: powers of two, exact) in every lane, from column l of the in-plane block
+// and entry l of the out-of-plane one (TrajP::detc in parts); gz = -2 gamma, qz = 1/(2 gamma)
+__device__ __forceinline__ Cx2<double> det8(double X0, double X1, double Y0, double Y1, double w, double gz, double qz,
+                                            int t, bool odd) {
+    const double X0p = xor_lane(X0, 2 * kT), X1p = xor_lane(X1, 2 * kT), Y0p = xor_lane(Y0, 2 * kT),
+                 Y1p = xor_lane(Y1, 2 * kT);   // column l + 2 in lanes 0 and 1
+    const double aq = from_lane(w, t), ap = from_lane(w, t + kT), bq = from_lane(w, t + 2 * kT),
+                 bp = from_lane(w, t + 3 * kT);
+    double zr0 = Y0p + X0, zr1 = Y1p + X1;
+    double zi0 = fma(gz, X0p, qz * Y0), zi1 = fma(gz, X1p, qz * Y1);
+    // column (l & 1) of Z in every lane, then both
+    zr0 = from_lane(zr0, t + odd * kT);
+    zr1 = from_lane(zr1, t + odd * kT);
+    zi0 = from_lane(zi0, t + odd * kT);
+    zi1 = from_lane(zi1, t + odd * kT);
+    const double wr0 = xor_lane(zr0, kT), wr1 = xor_lane(zr1, kT), wi0 = xor_lane(zi0, kT), wi1 = xor_lane(zi1, kT);
+    const double r00 = odd ? wr0 : zr0, r10 = odd ? wr1 : zr1, i00 = odd ? wi0 : zi0, i10 = odd ? wi1 : zi1;
+    const double r01 = odd ? zr0 : wr0, r11 = odd ? zr1 : wr1, i01 = odd ? zi0 : wi0, i11 = odd ? zi1 : wi1;
+    const double u1 = i00 * (odd ? r11 : i11), u2 = i01 * (odd ? r10 : i10);
+    const double dd = fma(r00, odd ? i11 : r11, odd ? u1 : -u1) - fma(r01, odd ? i10 : r10, odd ? u2 : -u2);
+    const double dx = xor_lane(dd, kT);
+    const double ar = odd ? dx : dd, ai = odd ? dd : dx;
+    // Z_yy: the real part in even and the imaginary part in odd lanes, then both
+    double y = fma(odd ? qz : 1.0, odd ? ap : bp, odd ? 0.0 : aq);
+    if (odd) y = fma(gz, bq, y);
+    const double yx = xor_lane(y, kT);
+    const double yr = odd ? yx : y, yi = odd ? y : yx;
+    const double u3 = ai * (odd ? yr : yi);
+    const double de = fma(ar, odd ? yi : yr, odd ? u3 : -u3);
+    const double df = xor_lane(de, kT);
+    return Cx2<double>{odd ? df : de, odd ? de : df};
+}
+
+// matrix: the step matrix of grid point n and the action's integrand at its stages
+template <int POT, bool FB>
 __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommon& cm, QShared& sm) {
     const PotConst<double> pc = pot_const<POT>(tg);
     const StepK<double> hk = f.k64;
@@ -173,9 +268,8 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
     auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(E + j) : 0.0; };
     const int e_off = l == 0 ? 0 : (l == 3 ? 2 : 1);   // stage l reads E at t, t + h/2, t + h/2, t + h
     double e_cur = e_at(2 * cm.n_first + e_off);
-    double S = 0.0;
-    Consumer in_q(0);
-    Producer out(1);
+    Consumer<2> in_q(kHand0);
+    Producer<2> out(kHand1);
     const double h = hk.h, c2 = hk.c2, c4 = hk.c4, c3 = hk.c3, c1 = hk.h6;
     for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
         const double e_next = e_at(2 * n + 2 + e_off);
@@ -186,9 +280,8 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
         const double x = st[0], z = st[kT], g = st[2 * kT], px = st[4 * kT], pz = st[5 * kT];
         double hs, V;
         if constexpr (POT == POT_SOFTCORE) {
-            const double s = st[3 * kT], s2 = s * s;
-            hs = -3.0 * g * s2;
-            V = -s;
+            hs = -3.0 * g * st[6 * kT];
+            V = -st[3 * kT];
         } else if constexpr (POT == POT_TONGLIN) {
             const double ir = st[3 * kT], Y = st[6 * kT], Y1 = st[7 * kT];
             const double r = fma(x, x, z * z) * ir;
@@ -225,21 +318,17 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
         o[(4 + l) * kT] = fma(-c3, s23, ei == ej ? h : 0.0);
         o[(8 + l) * kT] = fma(c3, p31 + p42, -c1 * (fma(2.0, s23, h0e) + h3e));
         o[(12 + l) * kT] = fma(c4, p42, -c2 * (s23 + h3e));
-        // out-of-plane rows: (a, b) in even lanes, (c, d) in odd lanes
-        const double g23 = g1 + g2;
-        const double ad = fma(c4, (odd ? g3 : g2) * (odd ? g1 : g0), -c2 * (g23 + (odd ? g3 : g0)));
-        const double w = fma(g2, g0, g3 * g1), v = -c1 * (fma(2.0, g23, g0) + g3);
-        const double bc = fma(odd ? c3 : -c3, odd ? w : g23, odd ? v : h);
-        if (l < 2) {
-            o[(kM + 2 * l) * kT] = odd ? bc : ad;
-            o[(kM + 2 * l + 1) * kT] = odd ? ad : bc;
+        if constexpr (FB) {
+            o[(kM + l) * kT] = l == 0 ? g0 : (l == 1 ? g1 : (l == 2 ? g2 : g3));
+        } else {
+            const double2 r = out_of_plane(hk, g0, g1, g2, g3, odd);
+            if (l < 2) {
+                o[(kM + 2 * l) * kT] = r.x;
+                o[(kM + 2 * l + 1) * kT] = r.y;
+            }
         }
         o[(kState + l) * kT] = state_l;
-        if (l == 0) o[kAct * kT] = S;   // the action at grid point n
-        // h/6 (k1 + 2 (k2 + k3) + k4)
-        const double k1 = from_lane(kS, t), k2 = from_lane(kS, t + kT), k3 = from_lane(kS, t + 2 * kT),
-                     k4 = from_lane(kS, t + 3 * kT);
-        if (cm.have && n >= cm.n0 && n < cm.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, c1);
+        o[(kAct + l) * kT] = kS;
         out.publish(dq);
         e_cur = e_next;
     }
@@ -247,78 +336,129 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
 }
 
 // columns: lane c advances column c of the in-plane block; lanes 0..3 hold
-// dy/dy0, dpy/dy0, dy/dpy0, dpy/dpy0 of the out-of-plane block
-__device__ void quad_columns(const QCommon& cm, QShared& sm) {
+// dy/dy0, dpy/dy0, dy/dpy0, dpy/dpy0 of the out-of-plane block; with FP64 bins also det Z
+// and its branch, with float bins (a light bins warp) the out-of-plane rows and the action
+template <int POT, bool FB>
+__device__ void quad_columns(const FieldDev& f, const TrajArgs& a, const QCommon& cm, QShared& sm) {
     const int t = cm.t, l = cm.l;
     const bool odd = l & 1;
+    const StepK<double> hk = f.k64;
+    const double gz = -2.0 * a.gamma, qz = 2.0 * a.qg64;
     double X0 = l == 0 ? 1.0 : 0.0, X1 = l == 1 ? 1.0 : 0.0, Y0 = l == 2 ? 1.0 : 0.0, Y1 = l == 3 ? 1.0 : 0.0;
     double w = (l == 0 || l == 3) ? 1.0 : 0.0;
+    Cx2<double> Dp{8.0, 0.0};
+    double sgn = 1.0;
+    unsigned turned = 0;   // the step into this grid point moved arg det Z by more than pi/2
+    double S = 0.0;        // the action at grid point n
     const volatile int* alive = sm.alive;
-    Consumer in_q(1);
-    Producer out(2);
+    Consumer<2> in_q(kHand1);
+    Producer<3> out(kHand2);
     for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
         const int di = in_q.wait();
         const double* const in = sm.s12[di] + t;
+        int dq = 0;
+        if constexpr (!FB) {
+            dq = out.acquire();
+            double* const o = sm.s23[dq] + t;
+            // 8 det Z at grid point n: re, im, the branch's sign (doubled after a turn)
+            if (l < 3) o[(kDetD + l) * kT] = l == 0 ? Dp.re : (l == 1 ? Dp.im : (turned ? 2.0 * sgn : sgn));
+            o[l * kT] = in[(kState + l) * kT];
+            o[(4 + l) * kT] = in[(kAct + l) * kT];
+            out.publish(dq);
+        }
+        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
         const double wp = xor_lane(w, kT);   // the other entry of this out-of-plane column
-        if (cm.have && n >= cm.n0 && n < cm.n_last && alive[t]) {
+        double m0, m1;
+        if constexpr (FB) {
+            const double2 r = out_of_plane(hk, in[kM * kT], in[(kM + 1) * kT], in[(kM + 2) * kT], in[(kM + 3) * kT], odd);
+            m0 = r.x;
+            m1 = r.y;
+        } else {
+            m0 = in[(kM + 2 * odd) * kT];
+            m1 = in[(kM + 2 * odd + 1) * kT];
+        }
+        if (step) {
             const double x0 = X0, x1 = X1, y0 = Y0, y1 = Y1;
             X0 = fma(in[0], x0, fma(in[kT], x1, fma(in[4 * kT], y0, fma(in[5 * kT], y1, x0))));
             X1 = fma(in[2 * kT], x0, fma(in[3 * kT], x1, fma(in[5 * kT], y0, fma(in[7 * kT], y1, x1))));
             Y0 = fma(in[8 * kT], x0, fma(in[9 * kT], x1, fma(in[12 * kT], y0, fma(in[13 * kT], y1, y0))));
             Y1 = fma(in[10 * kT], x0, fma(in[11 * kT], x1, fma(in[14 * kT], y0, fma(in[15 * kT], y1, y1))));
-            const double m0 = in[(kM + 2 * odd) * kT], m1 = in[(kM + 2 * odd + 1) * kT];
             const double q = odd ? wp : w, p = odd ? w : wp;
             w = fma(m0, q, fma(m1, p, w));
         }
-        const double state_l = in[(kState + l) * kT];
-        const double S = in[kAct * kT];
-        in_q.release(di);
-        const int dq = out.acquire();
-        double* const o = sm.s23[dq] + t;
-        o[(4 * l) * kT] = X0;
-        o[(4 * l + 1) * kT] = X1;
-        o[(4 * l + 2) * kT] = Y0;
-        o[(4 * l + 3) * kT] = Y1;
-        o[(16 + l) * kT] = w;
-        o[(20 + l) * kT] = state_l;
-        if (l == 0) o[24 * kT] = S;
-        out.publish(dq);
+        if constexpr (FB) {
+            const double state_l = in[(kState + l) * kT], s_n = S;
+            if (cm.have && n >= cm.n0 && n < cm.n_last)
+                S += TrajP<double, POT>::action_sum(in[kAct * kT], in[(kAct + 1) * kT], in[(kAct + 2) * kT],
+                                                    in[(kAct + 3) * kT], hk.h6);
+            in_q.release(di);
+            dq = out.acquire();
+            double* const o = sm.s23[dq] + t;
+            o[l * kT] = state_l;
+            if (l == 0) o[4 * kT] = s_n;
+            o[(kDetF + 4 * l) * kT] = X0;
+            o[(kDetF + 4 * l + 1) * kT] = X1;
+            o[(kDetF + 4 * l + 2) * kT] = Y0;
+            o[(kDetF + 4 * l + 3) * kT] = Y1;
+            o[(kDetF + 16 + l) * kT] = w;
+            out.publish(dq);
+        } else {
+            in_q.release(di);
+            const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, odd);
+            turned = 0;
+            if (step) follow_branch<double>(Dp, D, sgn, turned);
+        }
     }
     out.drain();
 }
 
-// bins: det Z and its branch, labels, removal, prefactor and the recombination sums
-template <int POT>
+// bins: labels, removal, prefactor and the recombination sums
+template <int POT, bool FB>
 __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms& gt, const TrajArgs& a,
                           const QCommon& c, QShared& sm) {
     const int t = c.t, l = c.l;
-    const bool odd = l & 1;
     const Cx<double> amp{c.have ? a.amp_re[c.i] : 0.0, c.have ? a.amp_im[c.i] : 0.0};
-    const bool fbins = a.float_bins != 0;   // recombination terms in float (as the float pass forms them)
     const float gamf = (float)a.gamma;
     bool alive = c.alive0;
     unsigned flags = (c.have && !alive) ? 8u : 0u;
-    Cx2<double> Dp{1.0, 0.0};
-    double sgn = 1.0;
-    const double hz = 0.5, gz = -a.gamma, qz = a.qg64;
     const bool pw = a.pw_mask != 0;
     const double pw_r2 = a.pw_radius * a.pw_radius;
     int pw_cls = -1;
     bool pw_in = false;
     unsigned long long all_steps = 0, steps = 0;
+    double S = 0.0;   // the action at grid point n
+    // float bins: 8 det Z and its branch
+    const double gz = -2.0 * a.gamma, qz = 2.0 * a.qg64;
+    Cx2<double> Dp{8.0, 0.0};
+    double sgn = 1.0;
     int rem = (int)(c.n_first % c.n_out);
     int64_t k_bin = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
-    Consumer in_q(2);
+    Consumer<3> in_q(kHand2);
     for (int64_t n = c.n_first; n <= c.n_last; ++n) {
         const int di = in_q.wait();
         const double* const in = sm.s23[di] + t;
-        const double X0 = in[(4 * l) * kT], X1 = in[(4 * l + 1) * kT], Y0 = in[(4 * l + 2) * kT],
-                     Y1 = in[(4 * l + 3) * kT];
-        const double aq = in[16 * kT], ap = in[17 * kT], bq = in[18 * kT], bp = in[19 * kT];
-        const double q0 = in[20 * kT], q2 = in[21 * kT], p0 = in[22 * kT], p2 = in[23 * kT], S = in[24 * kT];
+        const double q0 = in[0], q2 = in[kT], p0 = in[2 * kT], p2 = in[3 * kT];
+        double k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0;
+        double X0 = 0.0, X1 = 0.0, Y0 = 0.0, Y1 = 0.0, w = 0.0;
+        if constexpr (FB) {
+            S = in[4 * kT];
+            X0 = in[(kDetF + 4 * l) * kT];
+            X1 = in[(kDetF + 4 * l + 1) * kT];
+            Y0 = in[(kDetF + 4 * l + 2) * kT];
+            Y1 = in[(kDetF + 4 * l + 3) * kT];
+            w = in[(kDetF + 16 + l) * kT];
+        } else {
+            k1 = in[4 * kT];
+            k2 = in[5 * kT];
+            k3 = in[6 * kT];
+            k4 = in[7 * kT];
+            Dp = Cx2<double>{in[kDetD * kT], in[(kDetD + 1) * kT]};
+            sgn = in[(kDetD + 2) * kT];
+        }
         in_q.release(di);
         const bool on_bin = rem == 0;
+        if (!FB && alive && (__double2hiint(sgn) & 0x7fffffff) == 0x40000000) flags |= 4u;   // |sgn| = 2
         // partial waves (Sec. III.A-B), as in redo.cu
         if (pw && alive && n >= c.n0) {
             const double qx = q0, qy = 0.0, qzz = q2;
@@ -336,47 +476,59 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
             bool valid = false;
             Cx<double> C{0.0, 0.0};
             if (alive && n >= c.n0) {
+                const cd D = 0.125 * cd{Dp.re, Dp.im};
                 const double fs = q0 + q2 + p0 + p2;
                 const bool ok = isfinite(fs) && isfinite(S);
-                const cd D{Dp.re, Dp.im};
                 const double m2 = D.re * D.re + D.im * D.im;
                 if (!ok || !(m2 <= a.d_t * a.d_t)) {
                     alive = false;
                     flags |= 1u;
                     if (!ok || !isfinite(m2)) flags |= 2u;
                 } else if (n >= c.k_cnt && pw_ok) {
-                    cd Cz = c_sqrt(D);
+                    // principal root of det Z with |det Z| from m2 (D_t bounds it)
+                    const double r = sqrt(m2);
+                    const double q = sqrt(0.5 * (r + fabs(D.re))), o = positive(q) ? D.im / (2.0 * q) : 0.0;
+                    cd Cz = D.re >= 0.0 ? mk(q, o) : mk(fabs(o), copysign(q, D.im));
                     if (sgn < 0.0) Cz = -Cz;
                     C = Cx<double>{Cz.re, Cz.im};
                     valid = true;
                 }
             }
             if (__any_sync(0xffffffffu, valid)) {
-                const double tk = f.t_start + (double)n * f.dt;
-                double sn, cs, cl = 0.0, cv = 0.0;
-                sincos(fmod(tg.ip * tk, 2.0 * kPi), &sn, &cs);
-                if (fbins) {
+                double cl = 0.0, cv = 0.0;
+                if constexpr (FB) {
                     if (valid && l == 0) {
                         const FloatState fsn(q0, 0.0, q2, p0, 0.0, p2, S);
                         float fl, fv;
                         contribution<float>(fsn, gt, gamf, Cx<float>{(float)C.re, (float)C.im},
-                                            Cx<float>{(float)amp.re, (float)amp.im}, Cx<float>{(float)cs, (float)(-sn)},
-                                            fl, fv);
+                                            Cx<float>{(float)amp.re, (float)amp.im},
+                                            Cx<float>{(float)sm.phase[k_bin & 15][0], (float)sm.phase[k_bin & 15][1]}, fl, fv);
                         cl = (double)fl;
                         cv = (double)fv;
                     }
                 } else {
+                    // e^{-i Ip t} in even lanes and e^{i S} in odd lanes
+                    double sn, cs;
+                    sincos((l & 1) ? S : bin_phase(f, tg, n), &sn, &cs);
+                    const double sn_o = xor_lane(sn, kT), cs_o = xor_lane(cs, kT);   // lane 0: e^{i S}
                     // the GTO terms in four parts
                     const PView v(q0, q2, p0, p2, S);
                     double pp, qq, pq;
                     recomb_invariants<double>(v, pp, qq, pq);
+                    const float ppf = (float)pp, qqf = (float)qq;
+                    float most = -INFINITY;
+                    for (int j = l; j < gt.n; j += 4) most = fmaxf(most, gto_size(gt, ppf, qqf, j));
+                    most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, kT));
+                    most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, 2 * kT));
                     GtoSums<double> g{};
-                    if (valid)
-                        for (int j = l; j < gt.n; j += 4) gto_terms<double>(gt, pp, qq, pq, j, j + 1, g);
+                    for (int j = l; j < gt.n; j += 4)
+                        if (valid && !(gto_size(gt, ppf, qqf, j) < most - kGtoNothing))
+                            gto_terms<double>(gt, pp, qq, pq, j, j + 1, g);
                     auto fold = [](double& x) {
                         x += xor_lane(x, kT);
                         x += xor_lane(x, 2 * kT);
                     };
+                    __syncwarp();
                     fold(g.s0.re);
                     fold(g.s0.im);
                     fold(g.s1.re);
@@ -388,8 +540,10 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
                         fold(g.s3.im);
                     }
                     if (valid && l == 0)
-                        contribution_final<double>(v, gt, a.gamma, C, amp, Cx<double>{cs, -sn}, g, cl, cv);
+                        contribution_closed<double>(v, gt, a.gamma, C, amp, Cx<double>{cs, -sn}, Cx<double>{cs_o, sn_o},
+                                                    g, cl, cv);
                 }
+                __syncwarp();
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) {   // over the trajectories (lanes 0..7 hold them)
                     cl += xor_lane(cl, o);
@@ -404,29 +558,14 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
         }
         alive_out[t] = alive ? 1 : 0;
         rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
-        // the step n -> n + 1: det Z of the advanced columns (TrajP::detc in parts)
-        const double X0p = xor_lane(X0, 2 * kT), X1p = xor_lane(X1, 2 * kT), Y0p = xor_lane(Y0, 2 * kT),
-                     Y1p = xor_lane(Y1, 2 * kT);   // column l + 2 in lanes 0 and 1
-        double zr0 = hz * (Y0p + X0), zr1 = hz * (Y1p + X1);
-        double zi0 = fma(gz, X0p, qz * Y0), zi1 = fma(gz, X1p, qz * Y1);
-        // column (l & 1) of Z in every lane, then both
-        zr0 = from_lane(zr0, t + odd * kT);
-        zr1 = from_lane(zr1, t + odd * kT);
-        zi0 = from_lane(zi0, t + odd * kT);
-        zi1 = from_lane(zi1, t + odd * kT);
-        const double wr0 = xor_lane(zr0, kT), wr1 = xor_lane(zr1, kT), wi0 = xor_lane(zi0, kT), wi1 = xor_lane(zi1, kT);
-        const double r00 = odd ? wr0 : zr0, r10 = odd ? wr1 : zr1, i00 = odd ? wi0 : zi0, i10 = odd ? wi1 : zi1;
-        const double r01 = odd ? zr0 : wr0, r11 = odd ? zr1 : wr1, i01 = odd ? zi0 : wi0, i11 = odd ? zi1 : wi1;
-        const double u1 = i00 * (odd ? r11 : i11), u2 = i01 * (odd ? r10 : i10);
-        const double dd = fma(r00, odd ? i11 : r11, odd ? u1 : -u1) - fma(r01, odd ? i10 : r10, odd ? u2 : -u2);
-        const double dx = xor_lane(dd, kT);
-        const double ar = odd ? dx : dd, ai = odd ? dd : dx;
-        const double yr = hz * (bp + aq), yi = fma(gz, bq, qz * ap);
-        const double u3 = ai * (odd ? yr : yi);
-        const double de = fma(ar, odd ? yi : yr, odd ? u3 : -u3);
-        const double df = xor_lane(de, kT);
+        if constexpr (FB) {
+            // the step n -> n + 1: det Z of the advanced columns
+            const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, l & 1);
+            if (alive && n >= c.n0 && n < c.n_last) follow_branch<double>(Dp, D, sgn, flags);
+        } else {
+            if (c.have && n >= c.n0 && n < c.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, f.k64.h6);
+        }
         if (alive && n >= c.n0 && n < c.n_last) {
-            follow_branch<double>(Dp, Cx2<double>{odd ? df : de, odd ? de : df}, sgn, flags);
             ++all_steps;
             if (n >= c.k_cnt) ++steps;
         }
@@ -456,7 +595,7 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
 }
 
 // One group of 8 list entries (list positions 8 g .. 8 g + 7).
-template <int POT>
+template <int POT, bool FB>
 __device__ void quad_group(const FieldDev& f, const TargetDev& tg, const GtoTerms& gt, const TrajArgs& a, int64_t g,
                            int64_t n_list, QShared& sm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -490,13 +629,14 @@ __device__ void quad_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     if (warp == 0 && c.l == 0) sm.alive[c.t] = c.alive0 ? 1 : 0;
     __syncthreads();
     const int role = (warp + (int)(g & 3)) & 3;
-    if (role == 0) quad_dynamics<POT>(f, tg, a, c, sm);
-    else if (role == 1) quad_matrix<POT>(f, tg, c, sm);
-    else if (role == 2) quad_columns(c, sm);
-    else quad_bins<POT>(f, tg, gt, a, c, sm);
+    if (role == 0) quad_dynamics<POT, FB>(f, tg, a, c, sm);
+    else if (role == 1) quad_matrix<POT, FB>(f, tg, c, sm);
+    else if (role == 2) quad_columns<POT, FB>(f, a, c, sm);
+    else quad_bins<POT, FB>(f, tg, gt, a, c, sm);
 }
 
-template <int POT>
+// FB: recombination terms in float, as the float pass forms them (escalation lists)
+template <int POT, bool FB>
 __global__ void __launch_bounds__(kThreads, 3) quad_kernel(FieldDev f, TargetDev tg, GtoTerms gt, TrajArgs a) {
     __shared__ QShared sm;
     __shared__ long long s_g;
@@ -506,17 +646,18 @@ __global__ void __launch_bounds__(kThreads, 3) quad_kernel(FieldDev f, TargetDev
     for (;;) {
         const int64_t g = src.next(a, s_g);
         if (g < 0) break;
-        quad_group<POT>(f, tg, gt, a, g, n_list, sm);
+        quad_group<POT, FB>(f, tg, gt, a, g, n_list, sm);
         __syncthreads();   // every role has drained its hand-offs before the next group
     }
 }
 
 template <int POT>
 cudaError_t launch_pot(const FieldDev& f, const TargetDev& t, const GtoTerms& gt, const TrajArgs& a, cudaStream_t s) {
-    const int64_t most = std::min<int64_t>(a.n, a.count ? a.quad_limit : a.n);
-    const int64_t need = (most + kT - 1) / kT;
-    const int64_t blocks = a.redo_ctr ? std::min<int64_t>(need, (int64_t)a.redo_lists * 4) : need;
-    quad_kernel<POT><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
+    // with a plan: persistent, as many blocks as fit on every SM (3); without one: a block
+    // per group
+    const int64_t blocks = a.redo_ctr ? (int64_t)a.redo_lists * 3 : (a.n + kT - 1) / kT;
+    if (a.float_bins) quad_kernel<POT, true><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
+    else quad_kernel<POT, false><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
     return cudaGetLastError();
 }
 

@@ -11,12 +11,10 @@
 // block of 128 threads holds 32 trajectories (one per lane) and gives each of
 // its four warps about a quarter of the FP64 work of every step:
 //   dynamics  RK4 stages of (q, p) and the stage Hessian data,
-//   matrix    the step matrix [[A, B], [C, D]] (and its out-of-plane analogue),
-//   columns   the stability columns advanced by the step matrix, and the action
-//             increment (moved here from the matrix role, the one with the most
-//             FP64 work: a group alone on its SM then keeps 0.68 of the FP64
-//             units busy instead of 0.65),
-//   bins      det Z of the new columns and the branch of sqrt det Z, the
+//   matrix    the in-plane step matrix [[A, B], [C, D]],
+//   columns   the in-plane stability columns advanced by the step matrix, and the
+//             action increment,
+//   bins      the out-of-plane block, det Z and the branch of sqrt det Z, the
 //             partial-wave labels, removal and the prefactor at the bins, and
 //             the GTO recombination sums, spread over the steps between bins,
 //             with the warp reduction and the atomic bin update.
@@ -26,6 +24,13 @@
 // blocks resident on one SM spread over its four sub-partitions.  Removal is
 // decided by the bins warp; the warps ahead of it learn of it a few grid
 // points late and only skip work that no longer counts.
+//
+// Lists long enough to fill the chip at 32 trajectories a block come here (quad_limit);
+// then the FP64 instructions of all roles decide, 19 cycles of the SM each: 84, 79, 84 and
+// 44 per step (soft-core), of which the branch's comparisons on the bits of doubles and
+// 8 det Z of 2 Z (no halves) saved 15.  Measured, mixed H 8 cycles, 1e6 births (12,200
+// redone): 496 -> 473 ms; FP64 H 1600 nm 3 cycles, 20011 births: 471 ms with one thread per
+// trajectory, 242 ms here (271 ms with every GTO term of every bin).
 //
 // Each part runs the same device functions as the one-thread-per-trajectory
 // kernel (TrajP::stages_qp / action_term / action_sum, TrajP::step_matrix,
@@ -46,12 +51,15 @@ constexpr int kThreads = 128;     // four warps
 // dynamics -> matrix: stage positions (8), g (4), h (4), stage momenta 2..4 (6), stage
 // potentials (4), three unused words, state (q0, q2, p0, p2)
 constexpr int kS01 = 33;
-// matrix -> columns: 19 matrix entries, state (q0, q2, p0, p2), then the action
+// matrix -> columns: 15 matrix entries, g (4), state (q0, q2, p0, p2), then the action
 // increment's inputs: stage z of stages 2..4 (3), stage momenta of stages 2..4 (6),
 // stage potentials (4); the columns warp reads E itself (static shared memory stays
 // within 48 KB per block)
 constexpr int kS12 = 36;
-constexpr int kS23 = 25;          // columns -> bins: columns after the step (16 in-plane, 4 out-of-plane), state
+constexpr int kS23 = 25;          // columns -> bins: in-plane columns after the step (16), g of the stages (4), state
+
+// barrier bases of the three hand-offs
+constexpr int kHand0 = 1, kHand1 = 5, kHand2 = 9;
 
 struct Shared {
     double s01[2][kS01][kW];
@@ -85,7 +93,7 @@ __device__ void run_dynamics(const FieldDev& f, const TargetDev& tg, const TrajA
     auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(E + j) : 0.0; };
     double e0 = e_at(2 * c.n_first), e1 = e_at(2 * c.n_first + 1), e2 = e_at(2 * c.n_first + 2);
     const volatile int* alive = sm.alive;
-    Producer out(0);
+    Producer<2> out(kHand0);
     for (int64_t n = c.n_first; n <= c.n_last; ++n) {
         {
             const int d = out.acquire();
@@ -128,8 +136,8 @@ __device__ void run_dynamics(const FieldDev& f, const TargetDev& tg, const TrajA
 template <int POT>
 __device__ void run_matrix(const FieldDev& f, const Common& c, Shared& sm, int lane) {
     const StepK<double> hk = f.k64;
-    Consumer in_q(0);
-    Producer out(1);
+    Consumer<2> in_q(kHand0);
+    Producer<2> out(kHand1);
     for (int64_t n = c.n_first; n <= c.n_last; ++n) {
         {
             const int di = in_q.wait();
@@ -149,7 +157,9 @@ __device__ void run_matrix(const FieldDev& f, const Common& c, Shared& sm, int l
                 }
                 const StepMat<double> M = TrajP<double, POT>::step_matrix(qs, gs, hs, hk);
 #pragma unroll
-                for (int k = 0; k < 19; ++k) o[k * kW] = M.m[k];
+                for (int k = 0; k < 15; ++k) o[k * kW] = M.m[k];   // (its out-of-plane part is left out)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o[(15 + k) * kW] = gs[k];
                 // the action increment's inputs
 #pragma unroll
                 for (int k = 1; k < 4; ++k) {
@@ -177,8 +187,8 @@ __device__ void run_columns(const FieldDev& f, const Common& c, Shared& sm, int 
     Action<double> S;
     S.init();
     const volatile int* alive = sm.alive;
-    Consumer in_q(1);
-    Producer out(2);
+    Consumer<2> in_q(kHand1);
+    Producer<2> out(kHand2);
     for (int64_t n = c.n_first; n <= c.n_last; ++n) {
         {
             const int di = in_q.wait();
@@ -189,7 +199,9 @@ __device__ void run_columns(const FieldDev& f, const Common& c, Shared& sm, int 
             if (c.have && n >= c.n0 && n < c.n_last && alive[lane]) {
                 StepMat<double> M;
 #pragma unroll
-                for (int k = 0; k < 19; ++k) M.m[k] = in[k * kW];
+                for (int k = 0; k < 15; ++k) M.m[k] = in[k * kW];
+#pragma unroll
+                for (int k = 15; k < 19; ++k) M.m[k] = 0.0;   // the bins warp advances the out-of-plane block
                 T.apply_step_matrix(M);
             }
             if (c.have && n >= c.n0 && n < c.n_last) {
@@ -219,12 +231,8 @@ __device__ void run_columns(const FieldDev& f, const Common& c, Shared& sm, int 
                 o[(4 * k + 2) * kW] = T.Y[k][0];
                 o[(4 * k + 3) * kW] = T.Y[k][1];
             }
-            o[16 * kW] = T.aq;
-            o[17 * kW] = T.ap;
-            o[18 * kW] = T.bq;
-            o[19 * kW] = T.bp;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o[(20 + k) * kW] = in[(19 + k) * kW];
+            for (int k = 0; k < 8; ++k) o[(16 + k) * kW] = in[(15 + k) * kW];   // g of the stages, state
             o[24 * kW] = s_n;
             in_q.release(di);
             out.publish(dq);
@@ -246,9 +254,10 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
     T.init(0.0, 0.0, 0.0, 0.0, 0.0, 0.0);
     bool alive = c.alive0;
     unsigned flags = (c.have && !alive) ? 8u : 0u;
-    Cx2<double> Dp{1.0, 0.0};
+    Cx2<double> Dp{8.0, 0.0};               // 8 det Z (of 2 Z: powers of two, exact)
     double sgn = 1.0;
     const double rg = a.gamma;
+    const StepK<double> hk = f.k64;
     const bool pw = a.pw_mask != 0;
     const double pw_r2 = a.pw_radius * a.pw_radius;
     int pw_cls = -1;
@@ -259,13 +268,17 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
     int64_t k_bin = 0;
     int j_next = 0;
     double bq0 = 0, bq2 = 0, bp0 = 0, bp2 = 0, bS = 0, p2s = 0, q2s = 0, pqs = 0;
-    float p2f = 0.f, q2f = 0.f, pqf = 0.f;
+    float p2f = 0.f, q2f = 0.f, pqf = 0.f, most = 0.f;   // most: size of the largest GTO term (FP64 bins)
     Cx<double> C{0.0, 0.0};
     GtoSums<double> acc{};
     GtoSums<float> accf{};
     auto terms = [&](int j0, int j1) {
-        if (fbins) gto_terms<float>(gt, p2f, q2f, pqf, j0, j1, accf);
-        else gto_terms<double>(gt, p2s, q2s, pqs, j0, j1, acc);
+        if (fbins) {
+            gto_terms<float>(gt, p2f, q2f, pqf, j0, j1, accf);
+        } else {
+            for (int j = j0; j < j1; ++j)
+                if (!(gto_size(gt, p2f, q2f, j) < most - kGtoNothing)) gto_terms<double>(gt, p2s, q2s, pqs, j, j + 1, acc);
+        }
     };
     auto finish = [&]() {
         double cl = 0.0, cv = 0.0;
@@ -274,7 +287,7 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
             const int64_t nb = k_bin * c.n_out;
             const double tk = f.t_start + (double)nb * f.dt;
             double sn, cs;
-            sincos(fmod(tg.ip * tk, 2.0 * kPi), &sn, &cs);
+            sincos(fmod_2pi(tg.ip * tk), &sn, &cs);
             if (fbins) {
                 float fl, fv;
                 contribution_final<float>(FloatState(bq0, 0.0, bq2, bp0, 0.0, bp2, bS), gt, gamf,
@@ -304,7 +317,7 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
     int rem = (int)(c.n_first % c.n_out);
     int64_t k_next = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
-    Consumer in_q(2);
+    Consumer<2> in_q(kHand2);
     for (int64_t n = c.n_first; n <= c.n_last; ++n) {
         {
             const int di = in_q.wait();
@@ -331,14 +344,17 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                 if (alive && n >= c.n0) {
                     const double fs = q0 + q2 + p0 + p2;
                     const bool ok = isfinite(fs) && isfinite(S);
-                    const cd D{Dp.re, Dp.im};
+                    const cd D = 0.125 * cd{Dp.re, Dp.im};
                     const double m2 = D.re * D.re + D.im * D.im;
                     if (!ok || !(m2 <= a.d_t * a.d_t)) {
                         alive = false;
                         flags |= 1u;
                         if (!ok || !isfinite(m2)) flags |= 2u;
                     } else if (n >= c.k_cnt && pw_ok) {
-                        cd Cz = c_sqrt(D);
+                        // principal root of det Z with |det Z| from m2 (D_t bounds it)
+                        const double r = sqrt(m2);
+                        const double q = sqrt(0.5 * (r + fabs(D.re))), o = positive(q) ? D.im / (2.0 * q) : 0.0;
+                        cd Cz = D.re >= 0.0 ? mk(q, o) : mk(fabs(o), copysign(q, D.im));
                         if (sgn < 0.0) Cz = -Cz;
                         C = Cx<double>{Cz.re, Cz.im};
                         valid = true;
@@ -349,8 +365,13 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                         bS = S;
                         if (fbins)
                             recomb_invariants<float>(FloatState(bq0, 0.0, bq2, bp0, 0.0, bp2, bS), p2f, q2f, pqf);
-                        else
+                        else {
                             recomb_invariants<double>(PView(bq0, bq2, bp0, bp2, bS), p2s, q2s, pqs);
+                            p2f = (float)p2s;
+                            q2f = (float)q2s;
+                            most = -INFINITY;
+                            for (int j = 0; j < gt.n; ++j) most = fmaxf(most, gto_size(gt, p2f, q2f, j));
+                        }
                     }
                 }
                 k_bin = k_next++;
@@ -368,11 +389,18 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                     T.Y[k][0] = in[(4 * k + 2) * kW];
                     T.Y[k][1] = in[(4 * k + 3) * kW];
                 }
-                T.aq = in[16 * kW];
-                T.ap = in[17 * kW];
-                T.bq = in[18 * kW];
-                T.bp = in[19 * kW];
-                const Cx2<double> D = T.detc(0.5, -rg, a.qg64);
+                // the out-of-plane block, H_s = g_s (TrajP::step_matrix and apply_step_matrix)
+                const double g0 = in[16 * kW], g1 = in[17 * kW], g2 = in[18 * kW], g3 = in[19 * kW];
+                const double g23 = g1 + g2;
+                const double oa = fma(hk.c4, g2 * g0, -hk.c2 * (g23 + g0)), ob = fma(-hk.c3, g23, hk.h);
+                const double oc = fma(hk.c3, fma(g2, g0, g3 * g1), -hk.h6 * (fma(2.0, g23, g0) + g3));
+                const double od = fma(hk.c4, g3 * g1, -hk.c2 * (g23 + g3));
+                const double ya = T.aq, pa = T.ap, yb = T.bq, pb = T.bp;
+                T.aq = fma(oa, ya, fma(ob, pa, ya));
+                T.ap = fma(oc, ya, fma(od, pa, pa));
+                T.bq = fma(oa, yb, fma(ob, pb, yb));
+                T.bp = fma(oc, yb, fma(od, pb, pb));
+                const Cx2<double> D = T.detc(1.0, -2.0 * rg, 2.0 * a.qg64);
                 follow_branch<double>(Dp, D, sgn, flags);
                 ++all_steps;
                 if (n >= c.k_cnt) ++steps;
@@ -550,9 +578,9 @@ __global__ void __launch_bounds__(kThreads, 4) redo_kernel(FieldDev f, TargetDev
 
 template <int POT>
 cudaError_t launch_pot(const FieldDev& f, const TargetDev& t, const GtoTerms& gt, const TrajArgs& a, cudaStream_t s) {
-    // persistent: as many blocks as fit (4 per SM), each looping over groups
-    const int64_t need = (a.n + kW - 1) / kW;   // an upper bound on the groups (the count is on the device)
-    const int64_t blocks = a.redo_ctr ? std::min<int64_t>(need, (int64_t)a.redo_lists * 4) : need;
+    // with a plan: persistent, as many blocks as fit on every SM (4), each looping over the
+    // groups of its SM's list; without one: a block per group
+    const int64_t blocks = a.redo_ctr ? (int64_t)a.redo_lists * 4 : (a.n + kW - 1) / kW;
     redo_kernel<POT><<<(unsigned)blocks, kThreads, 0, s>>>(f, t, gt, a);
     return cudaGetLastError();
 }
@@ -578,12 +606,12 @@ int redo_lists() {
     return std::max(1, std::min(sms, kRedoLists));
 }
 
-// Longest list for the four-lane kernel, from FP64 instructions per step (64 cycles on
-// the longest role, 19 per SM for all roles): with m groups of 8 per SM it steps in
-// max(48 x 64, m x 135 x 19) cycles (soft-core), the 32-wide kernel with one group
-// per SM in about 7,600: two groups of 8 per SM win, three do not.  Tong-Lin: max(160
-// x 64, m x 265 x 19) against 24,000: four do.
-int64_t quad_limit(int pot, int lists) { return (int64_t)kQuadWidth * lists * (pot == POT_TONGLIN ? 4 : 2); }
+// Longest list for the four-lane kernel, from FP64 instructions per step (64 cycles each on
+// the longest role, 19 per SM for all roles): with m groups of 8 per SM it steps in about
+// max(2,900, m x 122 x 19) cycles (soft-core), the 32-wide kernel with one group per SM in
+// 6,400: two groups of 8 per SM win (4,600), three do not (7,000).  Tong-Lin: max(8,500, m
+// x 216 x 19) against 24,000: five do.
+int64_t quad_limit(int pot, int lists) { return (int64_t)kQuadWidth * lists * (pot == POT_TONGLIN ? 5 : 2); }
 
 cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;

@@ -18,11 +18,11 @@ struct PView {
     __device__ PView(double q0, double q2, double p0, double p2, double s) : q{q0, 0.0, q2}, p{p0, 0.0, p2}, S{s} {}
 };
 
-// Two-slot hand-offs between consecutive roles on named barriers (0 is left to
-// __syncthreads): hand-off h in {0, 1, 2}, slot d in {0, 1}; "full" is arrived at by
-// the producer and waited on by the consumer, "empty" the other way round, 64
-// threads each (the two warps).  A role runs ahead of the next by at most two
-// grid points, so uneven work per grid point evens out across the pipeline.
+// Hand-offs of N slots between consecutive roles on named barriers (0 is left to
+// __syncthreads): barrier base + d is "slot d full", arrived at by the producer and
+// waited on by the consumer, base + N + d "slot d empty", the other way round, 64 threads
+// each (the two warps).  A role runs ahead of the next by at most N grid points, so
+// uneven work per grid point evens out across the pipeline.
 // The barrier instructions want the warp converged.
 __device__ __forceinline__ void bar_sync64(int id) {
     __syncwarp();
@@ -32,35 +32,39 @@ __device__ __forceinline__ void bar_arrive64(int id) {
     __syncwarp();
     asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory");
 }
+template <int N>
 struct Producer {
-    int h;
+    int base, d;
+    bool wrapped;
     int64_t k;
-    __device__ explicit Producer(int h_) : h(h_), k(0) {}
-    __device__ int acquire() {                     // slot for item k, once its item k - 2 is consumed
-        const int d = (int)(k & 1);
-        if (k >= 2) bar_sync64(3 + 4 * h + d);
+    __device__ explicit Producer(int base_) : base(base_), d(0), wrapped(false), k(0) {}
+    __device__ int acquire() {                     // slot for item k, once its item k - N is consumed
+        if (wrapped) bar_sync64(base + N + d);
         return d;
     }
-    __device__ void publish(int d) {
-        bar_arrive64(1 + 4 * h + d);
+    __device__ void publish(int slot) {
+        bar_arrive64(base + slot);
         ++k;
+        if (++d == N) {
+            d = 0;
+            wrapped = true;
+        }
     }
     __device__ void drain() {                      // the consumer's releases of the last items
-        for (int64_t j = (k >= 2 ? k - 2 : 0); j < k; ++j) bar_sync64(3 + 4 * h + (int)(j & 1));
+        for (int64_t j = (k >= N ? k - N : 0); j < k; ++j) bar_sync64(base + N + (int)(j % N));
     }
 };
+template <int N>
 struct Consumer {
-    int h;
-    int64_t k;
-    __device__ explicit Consumer(int h_) : h(h_), k(0) {}
+    int base, d;
+    __device__ explicit Consumer(int base_) : base(base_), d(0) {}
     __device__ int wait() {
-        const int d = (int)(k & 1);
-        bar_sync64(1 + 4 * h + d);
+        bar_sync64(base + d);
         return d;
     }
-    __device__ void release(int d) {
-        bar_arrive64(3 + 4 * h + d);
-        ++k;
+    __device__ void release(int slot) {
+        bar_arrive64(base + N + slot);
+        if (++d == N) d = 0;
     }
 };
 
@@ -72,16 +76,23 @@ __device__ __forceinline__ unsigned sm_id() {
 
 // Where a block's next group of list entries comes from.  With a plan (redo_plan_kernel):
 // the groups of its own SM's list, longest first, then those left on the other lists,
-// one atomic counter per list.  Without one (a call that must not touch the shared
+// one atomic counter per list.  A block that finds its own list empty waits 20 us before
+// it turns to the others: the blocks of a launch start some microseconds apart, and a
+// second block on one SM would take the groups of SMs whose blocks are about to start
+// (groups of a short list then piled up on a few SMs: 167 to 220 ms for the same call).
+// SM s serves list (s + redo_shift) mod L: launches that run side by side (batches)
+// shift their lists, or the longest groups of all of them would meet on the first SMs.
+// Without one (a call that must not touch the shared
 // scratch): one group per block, rows of L blocks taken in alternating direction so
 // that a column of blocks (about one SM's) gets long and short groups.
 struct GroupSource {
     int probe, home;
+    bool waited;
     int64_t g_static;
-    __device__ GroupSource(const TrajArgs& a, int64_t n_groups) : probe(0), home(0), g_static(-1) {
+    __device__ GroupSource(const TrajArgs& a, int64_t n_groups) : probe(0), home(0), waited(false), g_static(-1) {
         const int L = a.redo_lists;
         if (a.redo_ctr) {
-            home = (int)(sm_id() % (unsigned)L);
+            home = (int)((sm_id() + (unsigned)a.redo_shift) % (unsigned)L);
         } else {
             const int64_t b = blockIdx.x, row = b / L, pos = b - row * L;
             const int64_t len = n_groups - row * L < L ? n_groups - row * L : L;
@@ -100,6 +111,10 @@ struct GroupSource {
         const int* const start = a.redo_ctr + 2 * kRedoLists;
         const int* const grp = a.redo_ctr + 3 * kRedoLists;
         for (; probe < L; ++probe) {
+            if (probe == 1 && !waited) {
+                waited = true;
+                __nanosleep(20000);
+            }
             const int l = (home + probe) % L;
             if (threadIdx.x == 0) {
                 const int k = atomicAdd(&a.redo_ctr[l], 1);

@@ -114,6 +114,7 @@ struct GtoTerms {
     // the same in float for the float recombination terms (no conversions in the loop)
     float kpf[kMaxGto], kqf[kMaxGto], kxf[kMaxGto], w0f[kMaxGto], w1f[kMaxGto], w2f[kMaxGto], w3f[kMaxGto];
     float nlf, nvf;
+    float lwf[kMaxGto];   // ln of the largest of |w0..w3| (-1e30 for a term without weight)
 };
 GtoTerms make_gto_terms(const TargetDev& t, double gamma);
 
@@ -168,6 +169,7 @@ struct TrajArgs {
     // clears them), then the plan that assigns the list's groups to the lists
     int redo_lists;
     int* redo_ctr;
+    int redo_shift;       // SM s serves group list (s + redo_shift) mod redo_lists
     int64_t quad_limit;   // lists up to this length run with four lanes per trajectory (quad.cu)
 };
 cudaError_t launch_traj(const FieldDev& f, const TargetDev& t, int precision, const TrajArgs& a,

@@ -95,6 +95,8 @@ GtoTerms make_gto_terms(const TargetDev& t, double gamma) {
         g.w1f[j] = (float)g.w1[j];
         g.w2f[j] = (float)g.w2[j];
         g.w3f[j] = (float)g.w3[j];
+        const double w = fmax(fmax(fabs(g.w0[j]), fabs(g.w1[j])), fmax(fabs(g.w2[j]), fabs(g.w3[j])));
+        g.lwf[j] = w > 0.0 ? (float)log(w) : -1e30f;
     }
     g.nlf = (float)g.nl;
     g.nvf = (float)g.nv;

@@ -118,11 +118,9 @@ __device__ __forceinline__ void potential_xz(R x, R z, const PotConst<R>& c, R& 
 // The fused operations are written out in the order that nvcc contracts potential_xz to in
 // the other FP64 kernels (found by comparing values over 1e6 positions): chaotic
 // trajectories follow the last bit of g, so the kernels agree only if every rounding does.
-__device__ __forceinline__ void tonglin_y(const PotConst<double>& c, double r, double e2, double e4, double e6,
-                                          double& Y, double& Y1) {
-    Y = fma(c.a5, e6, fma(c.a3 * r, e4, fma(c.a1, e2, c.Zc)));
-    Y1 = fma(-(c.a5 * c.a6), e6, fma(-c.a1 * c.a2t, e2, c.a3 * fma(-c.a4, r, 1.0) * e4));
-}
+//   Y  = fma(a5, e6, fma(a3 r, e4, fma(a1, e2, Zc))),
+//   Y' = fma(-a5 a6, e6, fma(-a1 a2, e2, (a3 fma(-a4, r, 1)) e4))
+// are formed in neighbouring lanes there.
 __device__ __forceinline__ double tonglin_g(double ir, double Y, double Y1) { return fma(Y, ir, -Y1) * (ir * ir); }
 __device__ __forceinline__ double tonglin_h(const PotConst<double>& c, double r, double ir, double Y, double Y1,
                                             double e2, double e4, double e6) {
@@ -841,6 +839,28 @@ __device__ __forceinline__ void follow_branch(Cx2<R>& Dp, Cx2<R> D, R& sgn, unsi
     Dp = D;
 }
 
+// x < 0 and x > 0 on the bits of a double: an FP64 comparison costs as much as an FP64
+// FMA on GB300, an integer one next to nothing
+__device__ __forceinline__ bool negative(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+__device__ __forceinline__ bool positive(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return b > 0ull && b <= 0x7ff0000000000000ull;
+}
+// the same in FP64 with 4 FP64 instructions instead of 9 (the sign of Dp.im D.im from its
+// factors)
+template <>
+__device__ __forceinline__ void follow_branch<double>(Cx2<double>& Dp, Cx2<double> D, double& sgn, unsigned& flags) {
+    const double cr = Dp.re * D.im - Dp.im * D.re;
+    const bool up = positive(Dp.im);
+    if (((up && negative(D.im)) || (negative(Dp.im) && positive(D.im))) && positive(cr) == up)
+        sgn = __hiloint2double(__double2hiint(sgn) ^ 0x80000000, __double2loint(sgn));
+    if (negative(Dp.re * D.re + Dp.im * D.im)) flags |= 4u;
+    Dp = D;
+}
+
 // range reduction to [-pi, pi] for the fast float sincos
 __device__ __forceinline__ float reduce_2pi(float x) {
     float k = rintf(x * 0.15915494309189535f);
@@ -904,9 +924,16 @@ __device__ __forceinline__ void gto_terms(const GtoTerms& gt, R p2, R q2, R pq, 
         }
     }
 }
+// Size of GTO term j in a recombination sum, as a logarithm: a term more than kGtoNothing
+// below the largest one is nothing beside it in 53 bits (e^{-60} < 1e-26), and an FP64 bin
+// leaves its exponential, sine and cosine (some 65 FP64 instructions) out.
+constexpr float kGtoNothing = 60.0f;
+__device__ __forceinline__ float gto_size(const GtoTerms& gt, float p2, float q2, int j) {
+    return fmaf(gt.kpf[j], p2, gt.kqf[j] * q2) + gt.lwf[j];
+}
 template <typename R, typename TT>
-__device__ __forceinline__ void contribution_final(const TT& T, const GtoTerms& gt, R gam, Cx<R> C, Cx<R> amp,
-                                                   Cx<R> eIp, const GtoSums<R>& a, R& out_l, R& out_v) {
+__device__ __forceinline__ void contribution_closed(const TT& T, const GtoTerms& gt, R gam, Cx<R> C, Cx<R> amp,
+                                                    Cx<R> eIp, Cx<R> eS, const GtoSums<R>& a, R& out_l, R& out_v) {
     const Cx<R> s0 = a.s0, s1 = a.s1, s2 = a.s2, s3 = a.s3;
     const R g = gam;
     const Cx<R> bz{R(2) * g * T.q[2], T.p[2]};          // 2 gamma q_z + i p_z
@@ -925,9 +952,7 @@ __device__ __forceinline__ void contribution_final(const TT& T, const GtoTerms& 
         dv = Cx<R>{-g * sv.im, g * sv.re};                 // i gamma * sv
     }
     // e^{i S} e^{-i Ip t_k} C amp
-    R ss, cc;
-    sc(T.S.reduced(), &ss, &cc);
-    Cx<R> P = cmul(cmul(Cx<R>{cc, ss}, eIp), cmul(C, amp));
+    Cx<R> P = cmul(cmul(eS, eIp), cmul(C, amp));
     Cx<R> cl = cmul(dl, P), cv = cmul(dv, P);
     if constexpr (std::is_same<R, float>::value) {
         out_l = -2.f * gt.nlf * cl.re;
@@ -936,6 +961,13 @@ __device__ __forceinline__ void contribution_final(const TT& T, const GtoTerms& 
         out_l = R(-2.0 * gt.nl) * cl.re;
         out_v = R(-2.0 * gt.nv) * cv.re;
     }
+}
+template <typename R, typename TT>
+__device__ __forceinline__ void contribution_final(const TT& T, const GtoTerms& gt, R gam, Cx<R> C, Cx<R> amp,
+                                                   Cx<R> eIp, const GtoSums<R>& a, R& out_l, R& out_v) {
+    R ss, cc;
+    sc(T.S.reduced(), &ss, &cc);
+    contribution_closed<R>(T, gt, gam, C, amp, eIp, Cx<R>{cc, ss}, a, out_l, out_v);
 }
 template <typename R, typename TT>
 __device__ __forceinline__ void contribution(const TT& T, const GtoTerms& gt, R gam, Cx<R> C,
@@ -955,6 +987,20 @@ template <>
 __device__ __forceinline__ const float* etable<float>(const FieldDev& f) { return f.E32; }
 __device__ __forceinline__ const double* etable_df(const FieldDev& f) { return f.E64; }
 
+// fmod(x, 2 pi) (2 pi as a double), the same value in a few FP64 instructions: the remainder
+// is a double, so one FMA with the right whole number of turns gives it exactly; the
+// product with 1/(2 pi) can be one turn off next to a multiple.
+__device__ __forceinline__ double fmod_2pi(double x) {
+    const double two_pi = 2.0 * kPi;
+    if (!(fabs(x) < 1e12)) return fmod(x, two_pi);
+    double n = trunc(x * 0.15915494309189535);
+    double r = fma(-n, two_pi, x);
+    const double one = copysign(1.0, x);
+    if (r * one < 0.0) r = fma(-(n - one), two_pi, x);
+    else if (fabs(r) >= two_pi) r = fma(-(n + one), two_pi, x);
+    return r;
+}
+
 // float view of an FP64 state for float recombination terms: coordinates rounded to
 // float, the action reduced mod 2 pi in FP64 and then rounded
 struct FloatState {
@@ -964,7 +1010,7 @@ struct FloatState {
         __device__ float reduced() const { return r; }
     } S;
     __device__ FloatState(double q0, double q1, double q2, double p0, double p1, double p2, double s)
-        : q{(float)q0, (float)q1, (float)q2}, p{(float)p0, (float)p1, (float)p2}, S{(float)fmod(s, 2.0 * kPi)} {}
+        : q{(float)q0, (float)q1, (float)q2}, p{(float)p0, (float)p1, (float)p2}, S{(float)fmod_2pi(s)} {}
 };
 
 // float view of a double-float trajectory for the recombination terms
