@@ -16,14 +16,19 @@
 // FMAs per time and bin instead of 6.  The Gaussian of a pair is
 //   e^{-delta^2/2s^2} e^{-(m dt)^2/2s^2} (e^{-delta dt/s^2})^{+-m},  delta = t_c - t_j:
 // one exponential per m for all times, and powers of a number near 1.  Block = 8 times
-// x 64 frequencies x 4 parts of the m range; the parts meet in shared memory.
+// x 64 frequencies x 4 parts of half of the m range; the parts meet in shared memory, the
+// halves (a cluster of two blocks) in the first block's.  Twice as many blocks even out
+// what the SMs get: 1300 blocks on 152 SMs are 9 at most for a mean of 8.6, 650 were 5
+// for 4.3 (1937 us).
 // Measured, 6620 bins, 400 times x 800 frequencies, windows of 2107 bins: 8387 us with a
-// rotation per time, frequency and bin, 1937 us now (8.4e8 FMAs: 1.4 ms).
+// rotation per time, frequency and bin, 1816 us now (8.4e8 FMAs: 1.4 ms).
 //
 // Emission time: a block of 16 warps per 32 frequencies scans |G(t_j, w)|^2 over the
 // analysis times in [t_a, t_b] for the centroid and the peak (vertex of the parabola
 // through ln|G|^2 at the maximum and its two neighbours); 122 -> 28 us at
 // the same size (one thread per frequency before).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "sfhk_device.cuh"
@@ -39,6 +44,7 @@ constexpr int kGThreads = 32 * kParts * kGroups;
 constexpr int kSpan = 64;           // m values between exact anchors of the rotation
 constexpr int kGTile = kParts * kSpan;
 
+constexpr int kHalves = 2;          // blocks of a cluster, along the m range
 static_assert(kGThreads == 2 * kTimes * 16 && kGThreads == kGTile, "one table entry and one m per thread");
 
 struct GaborShared {
@@ -51,11 +57,13 @@ struct GaborShared {
     long long m_lo, m_hi;
 };
 
-__global__ void __launch_bounds__(kGThreads)
+__global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
     gabor_kernel(const double* __restrict__ x, int64_t n_bins, double t0, double dt, double sigma,
                  const double* __restrict__ times, int64_t n_t, const double* __restrict__ omega, int64_t n_omega,
                  double* out_re, double* out_im) {
     __shared__ GaborShared sm;
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int half = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = warp % kParts, group = warp / kParts;
     const int64_t m_w = ((int64_t)blockIdx.x * kGroups + group) * 32 + lane;   // this lane's frequency
     const double w = m_w < n_omega ? omega[m_w] : 0.0;
@@ -94,8 +102,10 @@ __global__ void __launch_bounds__(kGThreads)
                     a = near < a ? near : a;
                     b = far > b ? far : b;
                 }
-            sm.m_lo = b < 0 ? 0 : a;
-            sm.m_hi = b;
+            // this block's half of it
+            const long long lo = b < 0 ? 0 : a, mid = lo + (b - lo + 1) / 2;
+            sm.m_lo = half ? mid : lo;
+            sm.m_hi = half ? b : mid - 1;
         }
         __syncthreads();
         const int64_t m_lo = sm.m_lo, m_hi = sm.m_hi;
@@ -144,19 +154,35 @@ __global__ void __launch_bounds__(kGThreads)
                 }
             }
         }
-        // the parts of the m range, in order, and e^{i w t_c}
+        // the parts of the m range, in order; the second block's sums go to the first one,
+        // into the place of its pairs
+        double2* const other = cluster.map_shared_rank(&sm.ab[0][0], 0);
+        double2 sum[kTimes];
 #pragma unroll
         for (int u = 0; u < kTimes; ++u) {
             __syncthreads();
             if (part > 0) sm.part[group][part - 1][lane] = make_double2(gr[u], gi[u]);
             __syncthreads();
-            if (part == 0 && jt + u < n_t && m_w < n_omega) {
-                double vr = gr[u], vi = gi[u];
+            if (part == 0) {
+                sum[u] = make_double2(gr[u], gi[u]);
                 for (int q = 0; q < kParts - 1; ++q) {
-                    vr += sm.part[group][q][lane].x;
-                    vi += sm.part[group][q][lane].y;
+                    sum[u].x += sm.part[group][q][lane].x;
+                    sum[u].y += sm.part[group][q][lane].y;
                 }
-                if (sm.lo[u] <= sm.hi[u]) {
+            }
+        }
+        cluster.sync();   // the first block has read its last tile
+        if (half == 1 && part == 0)
+#pragma unroll
+            for (int u = 0; u < kTimes; ++u) other[(u * kGroups + group) * 32 + lane] = sum[u];
+        cluster.sync();
+        if (half == 0 && part == 0 && m_w < n_omega) {
+#pragma unroll
+            for (int u = 0; u < kTimes; ++u) {
+                if (jt + u >= n_t) continue;
+                const double2 o = other[(u * kGroups + group) * 32 + lane];
+                double vr = sum[u].x + o.x, vi = sum[u].y + o.y;
+                if (sm.lo[u] <= sm.hi[u]) {   // times e^{i w t_c}
                     double s, c;
                     sincos(w * (t0 + (double)sm.c[u] * dt), &s, &c);
                     const double zr = fma(vr, c, -vi * s);
@@ -168,6 +194,7 @@ __global__ void __launch_bounds__(kGThreads)
             }
         }
     }
+    cluster.sync();   // no block leaves while the other may write to it
 }
 
 constexpr int kEWarps = 16;
@@ -251,7 +278,7 @@ cudaError_t launch_gabor(const double* bins, int64_t n_bins, double t0, double d
     if (n_omega == 0 || n_t == 0) return cudaSuccess;
     const unsigned gx = (unsigned)((n_omega + 32 * kGroups - 1) / (32 * kGroups));
     const unsigned gy = (unsigned)std::min<int64_t>((n_t + kTimes - 1) / kTimes, 65535);
-    gabor_kernel<<<dim3(gx, gy), kGThreads, 0, s>>>(bins, n_bins, t0, dt_out, sigma, times, n_t, omega, n_omega,
+    gabor_kernel<<<dim3(gx, gy, kHalves), kGThreads, 0, s>>>(bins, n_bins, t0, dt_out, sigma, times, n_t, omega, n_omega,
                                                     out_re, out_im);
     return cudaGetLastError();
 }
