@@ -660,7 +660,7 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
                 if (st) return st;
                 st = check_cuda(launch_compact(esc_bin + c0, cn, blk + blk_off, idx + c0, kfrom + c0, count + c, side),
                                 "compaction launch");
-                blk_off += compact_blocks(cn);
+                blk_off += compact_blocks(cn) + 1;   // (up to 8 chunks: the 16 words beyond the blocks hold them)
                 if (st) return st;
                 TrajArgs e = f;
                 e.esc_bin = nullptr;

@@ -3,7 +3,7 @@
 // escalation bins in [k_lo, k_hi], to the list
 // idx[0..count), k_from[0..count) in increasing birth index (hence n0) order,
 // so that the FP64 pass over the list keeps its blocks in lockstep.
-// Three launches: per-block counts, one-block exclusive scan, scatter.
+// Two launches: per-block counts, whose last block to finish scans them; scatter.
 #include "sfhk_internal.cuh"
 
 namespace sfhk {
@@ -30,22 +30,29 @@ __global__ void amp_max_kernel(const double* __restrict__ re, const double* __re
 
 __device__ __forceinline__ bool listed(int32_t e, int32_t k_lo, int32_t k_hi) { return e >= k_lo && e <= k_hi; }
 
-__global__ void count_kernel(const int32_t* __restrict__ esc, int64_t n, int32_t* blk, int32_t k_lo, int32_t k_hi) {
-    const int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x;
-    const int c = __syncthreads_count(i < n && listed(esc[i], k_lo, k_hi));
-    if (threadIdx.x == 0) blk[blockIdx.x] = c;
-}
-
-// exclusive scan of blk[0..nb) in place; total to *count
-__global__ void scan_kernel(int32_t* blk, int64_t nb, int32_t* count) {
+// Per-block counts into blk[0..nb); the last block to finish turns them into their
+// exclusive sums in place, the total into *count.  blk[nb] counts the finished blocks
+// (cleared before the launch).
+__global__ void count_kernel(const int32_t* __restrict__ esc, int64_t n, int32_t* blk, int64_t nb, int32_t* count,
+                             int32_t k_lo, int32_t k_hi) {
     __shared__ int32_t warp_tot[32];
     __shared__ int32_t carry;
-    if (threadIdx.x == 0) carry = 0;
+    __shared__ bool last;
+    const int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x;
+    const int c = __syncthreads_count(i < n && listed(esc[i], k_lo, k_hi));
+    if (threadIdx.x == 0) {
+        blk[blockIdx.x] = c;
+        __threadfence();   // the count is visible before the block counts as finished
+        last = atomicAdd(&blk[nb], 1) == (int32_t)(nb - 1);
+        carry = 0;
+    }
     __syncthreads();
+    if (!last) return;
+    __threadfence();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int64_t base = 0; base < nb; base += kB) {
         const int64_t k = base + threadIdx.x;
-        const int32_t v = k < nb ? blk[k] : 0;
+        const int32_t v = k < nb ? __ldcg(blk + k) : 0;
         int32_t x = v;   // inclusive warp scan
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -54,17 +61,8 @@ __global__ void scan_kernel(int32_t* blk, int64_t nb, int32_t* count) {
         }
         if (lane == 31) warp_tot[w] = x;
         __syncthreads();
-        if (w == 0) {
-            int32_t t = warp_tot[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int32_t y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
-            }
-            warp_tot[lane] = t;   // inclusive over warps
-        }
-        __syncthreads();
-        const int32_t before = carry + (w > 0 ? warp_tot[w - 1] : 0) + x - v;
+        int32_t before = carry + x - v;
+        for (int q = 0; q < w; ++q) before += warp_tot[q];
         if (k < nb) blk[k] = before;
         __syncthreads();
         if (threadIdx.x == kB - 1) carry = before + v;
@@ -108,8 +106,9 @@ cudaError_t launch_compact(const int32_t* esc_bin, int64_t n, int32_t* blk, int3
                            int32_t* count, cudaStream_t s, int32_t k_lo, int32_t k_hi) {
     const int64_t nb = compact_blocks(n);
     if (nb == 0) return cudaMemsetAsync(count, 0, sizeof(int32_t), s);
-    count_kernel<<<(unsigned)nb, kB, 0, s>>>(esc_bin, n, blk, k_lo, k_hi);
-    scan_kernel<<<1, kB, 0, s>>>(blk, nb, count);
+    const cudaError_t e = cudaMemsetAsync(blk + nb, 0, sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    count_kernel<<<(unsigned)nb, kB, 0, s>>>(esc_bin, n, blk, nb, count, k_lo, k_hi);
     scatter_kernel<<<(unsigned)nb, kB, 0, s>>>(esc_bin, n, blk, idx, k_from, k_lo, k_hi);
     return cudaGetLastError();
 }

@@ -217,6 +217,7 @@ inline cudaError_t launch_escalation(const FieldDev& f, const TargetDev& t, int 
     if (esc_precision == 1 && e.planar) return launch_traj(f, t, 2, e, s);
     return launch_traj(f, t, 0, e, s);
 }
+// blk: compact_blocks(n) + 1 ints of scratch
 cudaError_t launch_compact(const int32_t* esc_bin, int64_t n, int32_t* blk, int32_t* idx, int32_t* k_from,
                            int32_t* count, cudaStream_t s, int32_t k_lo = 0, int32_t k_hi = INT32_MAX);
 int64_t compact_blocks(int64_t n);
