@@ -31,12 +31,6 @@ __device__ __forceinline__ cd c_exp(cd z) {
     double e = exp(z.re);
     return cd{e * c, e * s};
 }
-// sin(x + i y) = sin x cosh y + i cos x sinh y
-__device__ __forceinline__ cd c_sin(cd z) {
-    double s, c;
-    sincos(z.re, &s, &c);
-    return cd{s * cosh(z.im), c * sinh(z.im)};
-}
 // cos(x + i y) = cos x cosh y - i sin x sinh y
 __device__ __forceinline__ cd c_cos(cd z) {
     double s, c;
