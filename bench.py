@@ -39,12 +39,12 @@ SM_MAX_MHZ = 2070.0
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the float pass
 # at the default configuration, per birth of the launch, from one full-size ncu capture of
 # the bench's own command (one pass, --clock-control none; the mean of its three launches:
-# 53,931,861 + 171 B for 1e6 births).  None while no capture of the kernel as it stands exists.
-FLOAT_PASS_DRAM_BYTES_PER_BIRTH = 53.932032
-# The same for the FP64 redo at the default configuration (6,989,739 + 0 B), keyed by
+# 53,672,363 + 1,963 B for 1e6 births).  None while no capture of the kernel as it stands exists.
+FLOAT_PASS_DRAM_BYTES_PER_BIRTH = 53.674325
+# The same for the FP64 redo at the default configuration (6,937,173 + 0 B), keyed by
 # (births, esc_ratio, esc_floor, esc_ratio_big, esc_big); other configurations, and
 # kernels changed since the capture, report null.
-REDO_DRAM_BYTES_DEFAULT = {(1_000_000, 200.0, 1e-2, 40.0, 1000.0): 6989739}
+REDO_DRAM_BYTES_DEFAULT = {(1_000_000, 200.0, 1e-2, 40.0, 1000.0): 6937173}
 
 
 # ----------------------------------------------------------------------------
@@ -86,9 +86,11 @@ def launches_per_step(n: int, n_steps: int, chunk: int, prec: int, floor: bool, 
     """Our kernels per step: births, the trajectory pass(es), spectra (x2).  The mixed
     path with escalation (as sfhk_dipole runs it) adds the amplitude maximum and, per
     birth chunk (overlap 0) or time segment (overlap 1) of the float pass, or once
-    (overlap 2, sequential), the float launch, three compaction kernels and the
-    high-precision redo (the four-warp redo of esc_precision 0, planar form, with its
-    one-warp group plan before it)."""
+    (overlap 2, sequential), the float launch, two compaction kernels and the
+    high-precision redo (esc_precision 0, planar form: its one-warp group plan and the
+    launches for short and for long lists, of which one returns at once).  One too many
+    per part where esc_precision is 1 or 2, and where a part has no more births than a
+    short list holds (only the launch for short lists follows)."""
     if prec != 1:
         return 1 + 1 + 2
     if overlap == 2:
