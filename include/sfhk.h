@@ -503,8 +503,9 @@ sfhk_status sfhk_spectrum(const double* bins, int64_t n_bins, double t0, double 
  * laser frequency, is the customary choice.
  * bins: device double[n_bins]; times: device double[n_times]; omega: device
  * double[n_omega]; out_re, out_im: device double[n_times * n_omega], row j
- * holds time t_j (overwritten).  SFHK_EINVAL for negative sizes, NULL arrays,
- * dt_out <= 0 or sigma <= 0 or non-finite.
+ * holds time t_j (overwritten; NaN where t_j is NaN and there are bins).
+ * SFHK_EINVAL for negative sizes, NULL arrays, dt_out <= 0 or sigma <= 0 or
+ * non-finite.
  * ---------------------------------------------------------------------- */
 sfhk_status sfhk_gabor(const double* bins, int64_t n_bins, double t0, double dt_out, double sigma,
                        const double* times, int64_t n_times, const double* omega, int64_t n_omega, double* out_re,

@@ -8,18 +8,20 @@
 // e^{-40} beyond).
 //
 // Bound by FP64 instructions (64 cycles of a sub-partition each on GB300), so the kernel
-// is built to need few per (time, frequency, bin).  About the bin c nearest to t_j the
-// windowed bins y of a pair c + m, c - m enter as
+// is built to need few per (time, frequency, bin).  About the window's bin c nearest to t_j
+// the windowed bins y of a pair c + m, c - m enter as
 //   e^{i w t_c} [ (y_{c+m} + y_{c-m}) cos(w m dt) + i (y_{c+m} - y_{c-m}) sin(w m dt) ]:
 // 2 FMAs a pair, and cos and sin depend on the frequency and m only, so a warp (one lane
 // per frequency) that holds 8 times forms them once for all 8: (16 + 4) / 16 = 1.25
 // FMAs per time and bin instead of 6.  The Gaussian of a pair is
 //   e^{-delta^2/2s^2} e^{-(m dt)^2/2s^2} (e^{-delta dt/s^2})^{+-m},  delta = t_c - t_j:
-// one exponential per m for all times, and powers of a number near 1.  Block = 8 times
-// x 64 frequencies x 4 parts of half of the m range; the parts meet in shared memory, the
-// halves (a cluster of two blocks) in the first block's.  Twice as many blocks even out
-// what the SMs get: 1300 blocks on 152 SMs are 9 at most for a mean of 8.6, 650 were 5
-// for 4.3 (1937 us).
+// one exponential per m for all times, and powers of one number per time (near 1 where
+// t_j lies among the bins).  The index arithmetic is in gabor_window.h: c stays within the
+// bins, so m and the work do too, and a time that is not a number takes no part in the sums
+// and has a row of NaN.  Block = 8 times x 64 frequencies x 4 parts of half of the m range;
+// the parts meet in shared memory, the halves (a cluster of two blocks) in the first
+// block's.  Twice as many blocks even out what the SMs get: 1300 blocks on 152 SMs are 9 at
+// most for a mean of 8.6, 650 were 5 for 4.3 (1937 us).
 // Measured, 6620 bins, 400 times x 800 frequencies, windows of 2107 bins: 8387 us with a
 // rotation per time, frequency and bin, 1816 us now (8.4e8 FMAs: 1.4 ms).
 //
@@ -31,12 +33,12 @@
 
 #include <algorithm>
 
+#include "gabor_window.h"
 #include "sfhk_device.cuh"
 
 namespace sfhk {
 namespace {
 
-constexpr double kGaborCut = 9.0;   // window half-width in units of sigma
 constexpr int kTimes = 8;           // analysis times per block
 constexpr int kParts = 4;           // parts of the m range (warps per 32 frequencies)
 constexpr int kGroups = 2;          // groups of 32 frequencies per block
@@ -74,38 +76,25 @@ __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
         __syncthreads();
         if (threadIdx.x < kTimes) {
             const int u = threadIdx.x;
-            // the bins of the window, none for a time past the end of the list
-            double lo = 1.0, hi = 0.0, tj = t0;
-            if (jt + u < n_t) {
-                tj = times[jt + u];
-                lo = fmax(ceil((tj - kGaborCut * sigma - t0) / dt), 0.0);
-                hi = fmin(floor((tj + kGaborCut * sigma - t0) / dt), (double)(n_bins - 1));
-            }
-            const bool any = lo <= hi;
-            // the bin nearest to t_j (it may lie beyond the bins)
-            const double c = any ? rint((tj - t0) / dt) : 0.0;
-            sm.c[u] = (long long)c;
-            sm.lo[u] = any ? (long long)lo : 1;
-            sm.hi[u] = any ? (long long)hi : 0;
-            const double d = any ? (t0 + c * dt) - tj : 0.0;
-            sm.delta[u] = d;
+            // no bins for a time past the end of the list
+            GaborWindow v{1, 0, 0, 0.0};
+            if (jt + u < n_t) v = gabor_window(times[jt + u], t0, dt, sigma, n_bins);
+            sm.c[u] = v.c;
+            sm.lo[u] = v.lo;
+            sm.hi[u] = v.hi;
+            sm.delta[u] = v.delta;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            // the m range of all eight windows
-            long long a = LLONG_MAX, b = -1;
-            for (int u = 0; u < kTimes; ++u)
-                if (sm.lo[u] <= sm.hi[u]) {
-                    const long long c = sm.c[u], l = sm.lo[u], h = sm.hi[u];
-                    const long long far = h - c > c - l ? h - c : c - l;
-                    const long long near = c < l ? l - c : (c > h ? c - h : 0);
-                    a = near < a ? near : a;
-                    b = far > b ? far : b;
-                }
-            // this block's half of it
-            const long long lo = b < 0 ? 0 : a, mid = lo + (b - lo + 1) / 2;
-            sm.m_lo = half ? mid : lo;
-            sm.m_hi = half ? b : mid - 1;
+            // this block's half of the m range of all eight windows
+            long long reach = -1;
+            for (int u = 0; u < kTimes; ++u) {
+                const long long r = gabor_reach(sm.lo[u], sm.hi[u], sm.c[u]);
+                reach = r > reach ? r : reach;
+            }
+            const long long mid = gabor_middle(reach);
+            sm.m_lo = half ? mid : 0;
+            sm.m_hi = half ? reach : mid - 1;
         }
         __syncthreads();
         const int64_t m_lo = sm.m_lo, m_hi = sm.m_hi;
@@ -188,6 +177,8 @@ __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
                     const double zr = fma(vr, c, -vi * s);
                     vi = fma(vr, s, vi * c);
                     vr = zr;
+                } else if (isnan(sm.delta[u])) {
+                    vr = vi = sm.delta[u];
                 }
                 out_re[(jt + u) * n_omega + m_w] = vr;
                 out_im[(jt + u) * n_omega + m_w] = vi;
