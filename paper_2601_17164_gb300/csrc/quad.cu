@@ -406,7 +406,7 @@ __device__ void quad_columns(const FieldDev& f, const TrajArgs& a, const QCommon
             in_q.release(di);
             const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, odd);
             turned = 0;
-            if (step) follow_branch<double>(Dp, D, sgn, turned);
+            if (step) follow_branch8(Dp, D, sgn, turned);
         }
     }
     out.drain();
@@ -485,10 +485,7 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
                     flags |= 1u;
                     if (!ok || !isfinite(m2)) flags |= 2u;
                 } else if (n >= c.k_cnt && pw_ok) {
-                    // principal root of det Z with |det Z| from m2 (D_t bounds it)
-                    const double r = sqrt(m2);
-                    const double q = sqrt(0.5 * (r + fabs(D.re))), o = positive(q) ? D.im / (2.0 * q) : 0.0;
-                    cd Cz = D.re >= 0.0 ? mk(q, o) : mk(fabs(o), copysign(q, D.im));
+                    cd Cz = root_det(D, m2);
                     if (sgn < 0.0) Cz = -Cz;
                     C = Cx<double>{Cz.re, Cz.im};
                     valid = true;
@@ -561,7 +558,7 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
         if constexpr (FB) {
             // the step n -> n + 1: det Z of the advanced columns
             const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, l & 1);
-            if (alive && n >= c.n0 && n < c.n_last) follow_branch<double>(Dp, D, sgn, flags);
+            if (alive && n >= c.n0 && n < c.n_last) follow_branch8(Dp, D, sgn, flags);
         } else {
             if (c.have && n >= c.n0 && n < c.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, f.k64.h6);
         }

@@ -351,10 +351,7 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                         flags |= 1u;
                         if (!ok || !isfinite(m2)) flags |= 2u;
                     } else if (n >= c.k_cnt && pw_ok) {
-                        // principal root of det Z with |det Z| from m2 (D_t bounds it)
-                        const double r = sqrt(m2);
-                        const double q = sqrt(0.5 * (r + fabs(D.re))), o = positive(q) ? D.im / (2.0 * q) : 0.0;
-                        cd Cz = D.re >= 0.0 ? mk(q, o) : mk(fabs(o), copysign(q, D.im));
+                        cd Cz = root_det(D, m2);
                         if (sgn < 0.0) Cz = -Cz;
                         C = Cx<double>{Cz.re, Cz.im};
                         valid = true;
@@ -401,7 +398,7 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                 T.bq = fma(oa, yb, fma(ob, pb, yb));
                 T.bp = fma(oc, yb, fma(od, pb, pb));
                 const Cx2<double> D = T.detc(1.0, -2.0 * rg, 2.0 * a.qg64);
-                follow_branch<double>(Dp, D, sgn, flags);
+                follow_branch8(Dp, D, sgn, flags);
                 ++all_steps;
                 if (n >= c.k_cnt) ++steps;
             }
