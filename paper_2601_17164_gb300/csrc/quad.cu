@@ -638,7 +638,9 @@ __global__ void __launch_bounds__(kThreads, 3) quad_kernel(FieldDev f, TargetDev
     __shared__ QShared sm;
     __shared__ long long s_g;
     const int64_t n_list = a.count ? (int64_t)*a.count : a.n;
-    if (a.count && n_list > a.quad_limit) return;   // a long list: redo.cu takes it
+    // an empty list (its blocks would otherwise look through every SM's list), or a long one,
+    // which redo.cu takes
+    if (a.count && (n_list == 0 || n_list > a.quad_limit)) return;
     GroupSource src(a, (n_list + kT - 1) / kT);
     for (;;) {
         const int64_t g = src.next(a, s_g);
