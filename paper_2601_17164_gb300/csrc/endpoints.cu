@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kThreads, 2) endpoints_kernel(FieldDev f, Targ
                 Eb = Fb;
                 Ec = Fc;
             }
-            __syncthreads();
+            if (__syncthreads_or(0)) break;
         }
     } else if (warp != 1) {
         // columns: warps 2..7 hold the derivatives to q0 (x, y, z) and p0 (x, y, z), at grid
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 2) endpoints_kernel(FieldDev f, Targ
                     }
                 }
             }
-            __syncthreads();
+            if (__syncthreads_or(0)) break;
         }
     } else {
         // det: grid point n - 2 in iteration n
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 2) endpoints_kernel(FieldDev f, Targ
                         ++steps;
                     }
                 }
-                bool write = u == n_last && have && !written;
+                bool write = false;
                 if ((rem == 0 || u == n_last) && live) {
                     const double fs = st[0][lane] + st[1][lane] + st[2][lane] + st[3][lane] + st[4][lane] + st[5][lane];
                     const bool ok = isfinite(fs) && isfinite(st[6][lane]);
@@ -248,6 +248,8 @@ __global__ void __launch_bounds__(kThreads, 2) endpoints_kernel(FieldDev f, Targ
                         Cacc = C;
                     }
                 }
+                // a trajectory that never started has its results at the end of the others
+                if (u == n_last || !__any_sync(0xffffffffu, alive)) write = have && !written;
                 if (write) {
                     written = true;
                     const size_t nn = (size_t)a.n;
@@ -269,7 +271,8 @@ __global__ void __launch_bounds__(kThreads, 2) endpoints_kernel(FieldDev f, Targ
                 }
                 rem = rem + 1 == n_out ? 0 : rem + 1;
             }
-            __syncthreads();
+            // every trajectory has its results: the block ends here
+            if (__syncthreads_or(__all_sync(0xffffffffu, written || !have))) break;
         }
         if (a.stats) {
             unsigned rm = __reduce_add_sync(0xffffffffu, (flags & 1u) ? 1u : 0u);

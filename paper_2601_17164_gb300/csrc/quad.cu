@@ -66,6 +66,7 @@ struct QShared {
     double hess[4 * 3 * kT];   // stage Hessians (a, b, c), matrix warp only
     double phase[16][2];       // cos and -sin of Ip t at bin k in row k & 15 (float bins)
     int alive[kT];             // written by the bins warp, read late by the warps ahead
+    long long last;            // the group's last grid point (GroupEnd)
 };
 
 struct QCommon {
@@ -164,8 +165,11 @@ __device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const Traj
     };
     int rem = (int)(cm.n_first % cm.n_out);
     int64_t k_bin = (cm.n_first + cm.n_out - 1) / cm.n_out;
-    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = cm.n_first; n <= end.last; ++n) {
         const int d = out.acquire();
+        const bool live = alive[t];
+        end.decide(n, live);
         // float bins: e^{-i Ip t} of the bin at this grid point (this warp has the FP64
         // instructions to spare; the hand-offs keep the bins warp less than 16 grid points
         // behind, so a row is read before its next use even with a bin at every point)
@@ -181,7 +185,7 @@ __device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const Traj
         rem = (rem + 1 == cm.n_out) ? 0 : rem + 1;
         double* const o = sm.s01[d] + t;
         const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
-        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
+        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && live;
         double g;
         const double qa = pair ? fma(hk.hh, p1, q1) : q1;                       // Q1, Q2
         const double ka = force(qa, pair ? e1 : e0, o + pair * kStage, g);      // F1, F2
@@ -271,9 +275,11 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
     Consumer<2> in_q(kHand0);
     Producer<2> out(kHand1);
     const double h = hk.h, c2 = hk.c2, c4 = hk.c4, c3 = hk.c3, c1 = hk.h6;
-    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = cm.n_first; n <= end.last; ++n) {
         const double e_next = e_at(2 * n + 2 + e_off);
         const int di = in_q.wait();
+        end.follow();
         const double* const in = sm.s01[di] + t;
         // stage l: Hessian data and the action integrand
         const double* const st = in + l * kStage;
@@ -353,8 +359,10 @@ __device__ void quad_columns(const FieldDev& f, const TrajArgs& a, const QCommon
     const volatile int* alive = sm.alive;
     Consumer<2> in_q(kHand1);
     Producer<3> out(kHand2);
-    for (int64_t n = cm.n_first; n <= cm.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = cm.n_first; n <= end.last; ++n) {
         const int di = in_q.wait();
+        end.follow();
         const double* const in = sm.s12[di] + t;
         int dq = 0;
         if constexpr (!FB) {
@@ -435,8 +443,10 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
     int64_t k_bin = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
     Consumer<3> in_q(kHand2);
-    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = c.n_first; n <= end.last; ++n) {
         const int di = in_q.wait();
+        end.follow();
         const double* const in = sm.s23[di] + t;
         const double q0 = in[0], q2 = in[kT], p0 = in[2 * kT], p2 = in[3 * kT];
         double k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0;
@@ -624,6 +634,7 @@ __device__ void quad_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     }
     c.n_first = m;
     if (warp == 0 && c.l == 0) sm.alive[c.t] = c.alive0 ? 1 : 0;
+    if (threadIdx.x == 0) sm.last = c.n_last;
     __syncthreads();
     const int role = (warp + (int)(g & 3)) & 3;
     if (role == 0) quad_dynamics<POT, FB>(f, tg, a, c, sm);

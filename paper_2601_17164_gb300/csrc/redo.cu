@@ -66,6 +66,7 @@ struct Shared {
     double s12[2][kS12][kW];
     double s23[2][kS23][kW];
     int alive[kW];   // written by the bins warp, read late and without order by the warps ahead
+    long long last;  // the group's last grid point (GroupEnd)
 };
 
 struct Common {
@@ -94,9 +95,12 @@ __device__ void run_dynamics(const FieldDev& f, const TargetDev& tg, const TrajA
     double e0 = e_at(2 * c.n_first), e1 = e_at(2 * c.n_first + 1), e2 = e_at(2 * c.n_first + 2);
     const volatile int* alive = sm.alive;
     Producer<2> out(kHand0);
-    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = c.n_first; n <= end.last; ++n) {
         {
             const int d = out.acquire();
+            const bool live = alive[lane];
+            end.decide(n, live);
             double* o = &sm.s01[d][0][lane];
             o[29 * kW] = T.q[0];
             o[30 * kW] = T.q[2];
@@ -104,7 +108,7 @@ __device__ void run_dynamics(const FieldDev& f, const TargetDev& tg, const TrajA
             o[32 * kW] = T.p[2];
             // the E values of the next step, loaded one step ahead
             const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
-            const bool step = c.have && n >= c.n0 && n < c.n_last && alive[lane];
+            const bool step = c.have && n >= c.n0 && n < c.n_last && live;
             if (step) {
                 double qs[4][2], gs[4], hs[4], ps[4][2], Vs[4];
                 T.stages_qp(e0, e1, e2, hk, pc, qs, gs, hs, ps, Vs);
@@ -138,9 +142,11 @@ __device__ void run_matrix(const FieldDev& f, const Common& c, Shared& sm, int l
     const StepK<double> hk = f.k64;
     Consumer<2> in_q(kHand0);
     Producer<2> out(kHand1);
-    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = c.n_first; n <= end.last; ++n) {
         {
             const int di = in_q.wait();
+            end.follow();
             const int dq = out.acquire();
             const double* in = &sm.s01[di][0][lane];
             double* o = &sm.s12[dq][0][lane];
@@ -189,9 +195,11 @@ __device__ void run_columns(const FieldDev& f, const Common& c, Shared& sm, int 
     const volatile int* alive = sm.alive;
     Consumer<2> in_q(kHand1);
     Producer<2> out(kHand2);
-    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = c.n_first; n <= end.last; ++n) {
         {
             const int di = in_q.wait();
+            end.follow();
             const int dq = out.acquire();
             const double* in = &sm.s12[di][0][lane];
             double* o = &sm.s23[dq][0][lane];
@@ -318,9 +326,11 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
     int64_t k_next = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
     Consumer<2> in_q(kHand2);
-    for (int64_t n = c.n_first; n <= c.n_last; ++n) {
+    GroupEnd end(sm.last);
+    for (int64_t n = c.n_first; n <= end.last; ++n) {
         {
             const int di = in_q.wait();
+            end.follow();
             const double* in = &sm.s23[di][0][lane];
             const double q0 = in[20 * kW], q2 = in[21 * kW], p0 = in[22 * kW], p2 = in[23 * kW], S = in[24 * kW];
             const bool on_bin = rem == 0;
@@ -469,6 +479,7 @@ __device__ void redo_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     }
     c.n_first = m;
     if (warp == 0) sm.alive[lane] = c.alive0 ? 1 : 0;
+    if (threadIdx.x == 0) sm.last = c.n_last;
     __syncthreads();
     const int role = (warp + (int)(g & 3)) & 3;
     if (role == 0) run_dynamics<POT>(f, tg, a, c, sm, lane);

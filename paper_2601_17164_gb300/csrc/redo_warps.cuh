@@ -93,6 +93,24 @@ struct Consumer {
     }
 };
 
+// The last grid point of a group, in shared memory: that of the call, until the bins warp
+// has removed every trajectory.  The dynamics warp, the first of the chain, learns of it
+// from the labels and makes the grid point that it is about to publish the last one; the
+// hand-offs order that write before the item, so each warp behind it reads it by the time
+// that it has waited for that item, and all four end on the same one.
+struct GroupEnd {
+    volatile long long* at;
+    int64_t last;
+    __device__ explicit GroupEnd(long long& shared) : at(&shared), last(shared) {}
+    __device__ void decide(int64_t n, bool alive) {   // by the dynamics warp, converged
+        if (!__any_sync(0xffffffffu, alive) && n < last) {
+            last = n;
+            if ((threadIdx.x & 31) == 0) *at = n;
+        }
+    }
+    __device__ void follow() { last = *at; }           // by the others, after the wait for an item
+};
+
 __device__ __forceinline__ unsigned sm_id() {
     unsigned r;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
