@@ -316,7 +316,9 @@ sfhk_status sfhk_resample_births(const sfhk_births* pool, int64_t m, int64_t n, 
  * dipole call in the planar form without deterministic bins runs on the
  * warp-specialised kernels of the escalation pass when block = chunk_steps = 0
  * (no scratch), FP64 endpoints on one of their own, and both with one thread
- * per trajectory otherwise.
+ * per trajectory otherwise and in calls so long that this is faster (endpoints
+ * of more than 416 births per SM in the Tong-Lin and 1088 in the other
+ * potentials, harmonic dipoles of more than 512).
  * chunk_steps: steps per shared-memory field window (0 = library choice;
  * else a multiple of n_out, 64..8192).
  * ---------------------------------------------------------------------- */

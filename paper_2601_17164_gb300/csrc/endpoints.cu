@@ -305,6 +305,14 @@ cudaError_t launch_pot(const FieldDev& f, const TargetDev& t, const TrajArgs& a,
 
 }  // namespace
 
+// Longest call for this kernel.  Where the one-thread kernel's warps fill the chip it needs
+// no hand-offs and no barriers, and its warps skip the steps after their last removal, of
+// which Tong-Lin trajectories have many (27 % below).  Measured, one-thread over this
+// kernel's time (800 nm 1 cycle, d_t 1e30, 152 SMs): soft-core 1.01 at 160,000, 0.99 at
+// 180,000, 0.98 at 400,000; harmonic 1.00 at 156,000 and 200,000; Tong-Lin 1.05 at 60,000,
+// 0.99 at 66,000, 0.85 at 100,000.
+int64_t endpoints_limit(int pot, int sms) { return (int64_t)kW * sms * (pot == POT_TONGLIN ? 13 : 34); }
+
 cudaError_t launch_endpoints(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     switch (t.pot) {

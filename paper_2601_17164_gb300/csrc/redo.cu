@@ -621,6 +621,13 @@ int redo_lists() {
 // x 216 x 19) against 24,000: five do.
 int64_t quad_limit(int pot, int lists) { return (int64_t)kQuadWidth * lists * (pot == POT_TONGLIN ? 5 : 2); }
 
+// Longest FP64 dipole call for the warp-specialised kernels.  The harmonic force leaves the
+// bins warp with most of the work, and the one-thread kernel is even from 80,000 births on
+// 152 SMs and faster beyond: its time over the 32-wide kernel's is 1.36 at 50,000, 1.00 at
+// 80,000, 0.98 at 100,000, 0.96 at 1e6; soft-core 1.05, Tong-Lin 1.01 and free 1.07 at 1e6
+// (800 nm, 1 cycle).
+int64_t fp64_limit(int pot, int sms) { return pot == POT_HARMONIC ? (int64_t)kW * sms * 16 : INT64_MAX; }
+
 cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     if (a.redo_lists < 1 || a.redo_lists > kRedoLists) return cudaErrorInvalidValue;

@@ -174,7 +174,9 @@ struct TrajArgs {
 };
 cudaError_t launch_traj(const FieldDev& f, const TargetDev& t, int precision, const TrajArgs& a,
                         cudaStream_t s);
-// FP64 endpoints of the full state, eight warps per 32 trajectories (endpoints.cu)
+// FP64 endpoints of the full state, eight warps per 32 trajectories (endpoints.cu), and the
+// longest call it takes
+int64_t endpoints_limit(int pot, int sms);
 cudaError_t launch_endpoints(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
 // 32-bit words of saved state per birth in a segmented float pass (planar or 3D form)
 int state_words(int planar);
@@ -199,7 +201,9 @@ inline size_t redo_scratch_words(int64_t n, int64_t quad_limit) {
     return 3 * (size_t)kRedoLists + 2 * (size_t)redo_groups(n, quad_limit);
 }
 cudaError_t launch_quad(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
-// the FP64 planar dipole of births [0, n) by the same kernels, without escalation list or scratch
+// the FP64 planar dipole of births [0, n) by the same kernels, without escalation list or
+// scratch, up to the longest call they take
+int64_t fp64_limit(int pot, int sms);
 cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
 int64_t redo_blocks(int64_t n);
 // The high-precision pass over an escalation list: esc_precision 0 FP64 (the split
