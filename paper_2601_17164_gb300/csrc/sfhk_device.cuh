@@ -160,4 +160,21 @@ __device__ __forceinline__ FieldAt0 field_at_real(const FieldDev& f, double t, c
     return r;
 }
 
+// sr + i si += sum over u < n of y[u] e^{i w t_{k0 + u}}, t_k = t0 + k dt, by a rotation per
+// bin (rc + i rs = e^{i w dt}) that an exact sincos re-anchors every 64 bins: the sum of the
+// transforms' short forms (spectrum.cu, gabor.cu)
+__device__ __forceinline__ void direct_sum(const double* y, int n, double w, double t0, double dt, int64_t k0,
+                                           double rc, double rs, double& sr, double& si) {
+    double er = 0.0, ei = 0.0;
+    for (int u = 0; u < n; ++u) {
+        if ((u & 63) == 0) sincos(w * (t0 + (double)(k0 + u) * dt), &ei, &er);
+        const double v = y[u];
+        sr = fma(v, er, sr);
+        si = fma(v, ei, si);
+        const double nr = fma(er, rc, -ei * rs);
+        ei = fma(er, rs, ei * rc);
+        er = nr;
+    }
+}
+
 }  // namespace sfhk

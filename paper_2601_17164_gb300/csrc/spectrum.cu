@@ -17,6 +17,12 @@
 // blocks, 111 us now (the pairs' FMAs alone take 45 us on all sub-partitions).  4 us of
 // them carry the phases' roundings (anchor): relative error against 64 bits, the worst
 // output, 8.6e-14; 2.7e-13 without, 1.4e-13 with one thread per frequency.
+//
+// Few bins (direct_bins): one thread per frequency with a rotation per bin.  The factors,
+// anchors and cluster barriers above take 24 us however few the bins (10 bins x 20: 24 us
+// against 9 us), and a warp's ~140 FP64 instructions for them in 16 warps per 32
+// frequencies outweigh the pairs where frequencies are many (500 bins x 2e5: 1.9 ms
+// against 1.25 ms).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -42,6 +48,40 @@ __device__ __forceinline__ void anchor(double w, double t0, double dt, int64_t k
     sincos(p, &sp, &cp);
     *s = fma(cp, e, sp);
     *c = fma(-sp, e, cp);
+}
+
+constexpr int kDirectTile = 1024;
+
+__global__ void spectrum_direct_kernel(const double* __restrict__ x, int64_t n_bins, double t0, double dt, double tau,
+                                       const double* __restrict__ omega, int64_t n_omega, double* out_re,
+                                       double* out_im) {
+    __shared__ double sx[kDirectTile];
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const double w = m < n_omega ? omega[m] : 0.0;
+    double sr = 0.0, si = 0.0, rs, rc;
+    sincos(w * dt, &rs, &rc);
+    for (int64_t k0 = 0; k0 < n_bins; k0 += kDirectTile) {
+        const int nt = (int)(n_bins - k0 < kDirectTile ? n_bins - k0 : kDirectTile);
+        __syncthreads();
+        for (int u = threadIdx.x; u < nt; u += blockDim.x) {
+            const double t = t0 + (double)(k0 + u) * dt;
+            const double W = fabs(t) <= tau ? 0.5 * (1.0 + cospi(t / tau)) : 0.0;
+            sx[u] = x[k0 + u] * W * dt;
+        }
+        __syncthreads();
+        direct_sum(sx, nt, w, t0, dt, k0, rc, rs, sr, si);
+    }
+    if (m < n_omega) {
+        out_re[m] = sr;
+        out_im[m] = si;
+    }
+}
+
+// Most bins for that kernel, where its time meets the other one's (152 SMs; its time over
+// the other's): up to 1200 frequencies 0.87 at 64 bins, 1.25 at 100; 5000: 0.93 at 200, 1.14
+// at 256; 20000: 0.97 at 400, 1.23 at 552; 1e5: 0.76 at 552, 1.14 at 1000.
+int64_t direct_bins(int64_t n_omega) {
+    return std::max<int64_t>(80, std::min<int64_t>(n_omega / 24, 400 + n_omega / 400));
 }
 
 __global__ void __launch_bounds__(32 * kMaxWarps)
@@ -179,6 +219,12 @@ cudaError_t launch_spectrum(const double* bins, int64_t n_bins, double t0, doubl
                             const double* omega, int64_t n_omega, double* out_re, double* out_im,
                             cudaStream_t s) {
     if (n_omega == 0) return cudaSuccess;
+    if (n_bins <= direct_bins(n_omega)) {
+        const int block = 128;
+        spectrum_direct_kernel<<<(unsigned)((n_omega + block - 1) / block), block, 0, s>>>(
+            bins, n_bins, t0, dt_out, tau_h, omega, n_omega, out_re, out_im);
+        return cudaGetLastError();
+    }
     // Blocks per group of 32 frequencies: as many as bring the grid to one block on each of
     // 152 SMs, at least 4 (16 warps: the parts' anchors still cost a tenth of the sums) and
     // at most 8 (the portable cluster size), those with 8 warps where even that leaves half
