@@ -25,6 +25,10 @@
 // Measured, 6620 bins, 400 times x 800 frequencies, windows of 2107 bins: 8387 us with a
 // rotation per time, frequency and bin, 1816 us now (8.4e8 FMAs: 1.4 ms).
 //
+// Short windows and few bins (direct_is_faster): one thread per frequency and time with a
+// rotation per bin, as the eight times' tables and the cluster's barriers take 21 to 28 us
+// however short the window.
+//
 // Emission time: a block of 16 warps per 32 frequencies scans |G(t_j, w)|^2 over the
 // analysis times in [t_a, t_b] for the centroid and the peak (vertex of the parabola
 // through ln|G|^2 at the maximum and its two neighbours); 122 -> 28 us at
@@ -56,8 +60,56 @@ struct GaborShared {
     double in_run[2][kTimes][16];             // dt e^{-delta^2/2s^2} e^{-+ b delta dt/s^2}
     double delta[kTimes];                     // t_c - t_j
     long long c[kTimes], lo[kTimes], hi[kTimes];
-    long long m_lo, m_hi;
+    long long reach, m_lo, m_hi;
 };
+
+constexpr int kDirectTile = 1024;
+
+// block = one analysis time x 128 frequencies
+__global__ void gabor_direct_kernel(const double* __restrict__ x, int64_t n_bins, double t0, double dt, double sigma,
+                                    const double* __restrict__ times, int64_t n_t, const double* __restrict__ omega,
+                                    int64_t n_omega, double* out_re, double* out_im) {
+    __shared__ double sx[kDirectTile];
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const double w = m < n_omega ? omega[m] : 0.0;
+    double rs, rc;
+    sincos(w * dt, &rs, &rc);
+    const double inv2s2 = 1.0 / (2.0 * sigma * sigma);
+    for (int64_t j = blockIdx.y; j < n_t; j += gridDim.y) {
+        const double tj = times[j];
+        const GaborBins v = gabor_bins(tj, t0, dt, sigma, n_bins);
+        double sr = 0.0, si = 0.0;
+        for (int64_t k0 = v.lo; k0 <= v.hi; k0 += kDirectTile) {
+            const int nt = (int)(v.hi - k0 + 1 < kDirectTile ? v.hi - k0 + 1 : kDirectTile);
+            __syncthreads();
+            for (int u = threadIdx.x; u < nt; u += blockDim.x) {
+                const double d = (t0 + (double)(k0 + u) * dt) - tj;
+                sx[u] = x[k0 + u] * exp(-d * d * inv2s2) * dt;
+            }
+            __syncthreads();
+            direct_sum(sx, nt, w, t0, dt, k0, rc, rs, sr, si);
+        }
+        if (m < n_omega) {
+            out_re[j * n_omega + m] = v.nan ? tj : sr;
+            out_im[j * n_omega + m] = v.nan ? tj : si;
+        }
+    }
+}
+
+// The faster kernel for a call, by what their times in microseconds were found to be on 152
+// SMs (windows of W bins, reach R of the pairs): the larger of one block's latency and of the
+// chip's throughput.  Measured against this estimate's choice, direct and blocked: 10 times x
+// 20 frequencies, W 91: 28 and 36, W 217: 58 and 46; 400 x 800, W 19: 136 and 181, W 55: 275
+// and 205; 100 bins under a window of 1054, 100 x 100: 31 and 44, 400 x 800: 474 and 267.
+bool direct_is_faster(int64_t n_bins, double half_width, int64_t n_t, int64_t n_omega) {
+    if (n_bins < 1) return true;
+    const double R = std::min((double)(n_bins - 1), half_width), W = std::min((double)n_bins, 2.0 * half_width + 1.0);
+    const double direct_pairs = (double)n_t * (double)((n_omega + 127) / 128 * 128);
+    const double blocked_pairs = (double)((n_t + 7) / 8 * 8) * (double)((n_omega + 63) / 64 * 64);
+    const double direct = std::max(8.5 + 0.216 * W, direct_pairs * (1.9e-4 + 1.08e-5 * W));
+    const double blocked = std::max((n_t < 8 ? 20.5 : 27.5) + 0.18 * R, blocked_pairs * (4.7e-4 + 4.9e-6 * R));
+    return direct <= blocked;
+}
 
 __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
     gabor_kernel(const double* __restrict__ x, int64_t n_bins, double t0, double dt, double sigma,
@@ -70,8 +122,6 @@ __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
     const int64_t m_w = ((int64_t)blockIdx.x * kGroups + group) * 32 + lane;   // this lane's frequency
     const double w = m_w < n_omega ? omega[m_w] : 0.0;
     const double inv2s2 = 1.0 / (2.0 * sigma * sigma);
-    double rs, rc;
-    sincos(w * dt, &rs, &rc);   // rotation per bin
     for (int64_t jt = (int64_t)blockIdx.y * kTimes; jt < n_t; jt += (int64_t)gridDim.y * kTimes) {
         __syncthreads();
         if (threadIdx.x < kTimes) {
@@ -93,11 +143,20 @@ __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
                 reach = r > reach ? r : reach;
             }
             const long long mid = gabor_middle(reach);
+            sm.reach = reach;
             sm.m_lo = half ? mid : 0;
             sm.m_hi = half ? reach : mid - 1;
         }
         __syncthreads();
+        if (sm.reach < 0) {   // no bins for any of the times (in both blocks of the cluster)
+            if (half == 0 && m_w < n_omega)
+                for (int u = part; u < kTimes && jt + u < n_t; u += kParts)   // (0, or NaN)
+                    out_re[(jt + u) * n_omega + m_w] = out_im[(jt + u) * n_omega + m_w] = sm.delta[u];
+            continue;
+        }
         const int64_t m_lo = sm.m_lo, m_hi = sm.m_hi;
+        double rs, rc;
+        sincos(w * dt, &rs, &rc);   // rotation per bin
         // this thread's entry of the two tables: side, time, place in the run or run
         const int e_side = threadIdx.x >> 7, e_u = (threadIdx.x >> 4) & (kTimes - 1), e_b = threadIdx.x & 15;
         const double e_d = sm.delta[e_u], theta = (e_side ? 2.0 : -2.0) * dt * e_d * inv2s2;
@@ -267,6 +326,13 @@ cudaError_t launch_gabor(const double* bins, int64_t n_bins, double t0, double d
                          const double* times, int64_t n_t, const double* omega, int64_t n_omega, double* out_re,
                          double* out_im, cudaStream_t s) {
     if (n_omega == 0 || n_t == 0) return cudaSuccess;
+    if (direct_is_faster(n_bins, floor(kGaborCut * sigma / dt_out), n_t, n_omega)) {
+        const int block = 128;
+        const dim3 grid((unsigned)((n_omega + block - 1) / block), (unsigned)std::min<int64_t>(n_t, 65535));
+        gabor_direct_kernel<<<grid, block, 0, s>>>(bins, n_bins, t0, dt_out, sigma, times, n_t, omega, n_omega, out_re,
+                                                   out_im);
+        return cudaGetLastError();
+    }
     const unsigned gx = (unsigned)((n_omega + 32 * kGroups - 1) / (32 * kGroups));
     const unsigned gy = (unsigned)std::min<int64_t>((n_t + kTimes - 1) / kTimes, 65535);
     gabor_kernel<<<dim3(gx, gy, kHalves), kGThreads, 0, s>>>(bins, n_bins, t0, dt_out, sigma, times, n_t, omega, n_omega,

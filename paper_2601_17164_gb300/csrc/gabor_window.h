@@ -16,26 +16,38 @@ namespace sfhk {
 
 constexpr double kGaborCut = 9.0;   // window half-width in units of sigma
 
-// Bins [lo, hi] of a time's window (none when lo > hi), its reference bin c in [lo, hi] and
-// delta = t_c - t_j.  delta is NaN for a time that is not a number: no bins, a row of NaN.
+// Bins [lo, hi] of a time's window, none when lo > hi.  A time that is not a number has no
+// bins, and a row of NaN (where there are bins at all).
+struct GaborBins {
+    long long lo, hi;
+    bool nan;
+};
+SFHK_HD GaborBins gabor_bins(double tj, double t0, double dt, double sigma, long long n_bins) {
+    GaborBins w{1, 0, false};
+    if (n_bins < 1) return w;
+    if (tj != tj) {
+        w.nan = true;
+        return w;
+    }
+    const double lo = fmax(ceil((tj - kGaborCut * sigma - t0) / dt), 0.0);
+    const double hi = fmin(floor((tj + kGaborCut * sigma - t0) / dt), (double)(n_bins - 1));
+    if (lo <= hi) {
+        w.lo = (long long)lo;
+        w.hi = (long long)hi;
+    }
+    return w;
+}
+// the same with the window's bin c nearest to the time and delta = t_c - t_j (NaN for a time
+// that is not a number, 0 without bins)
 struct GaborWindow {
     long long lo, hi, c;
     double delta;
 };
 SFHK_HD GaborWindow gabor_window(double tj, double t0, double dt, double sigma, long long n_bins) {
-    GaborWindow w{1, 0, 0, 0.0};
-    if (n_bins < 1) return w;
-    if (tj != tj) {
-        w.delta = tj;
-        return w;
-    }
-    const double lo = fmax(ceil((tj - kGaborCut * sigma - t0) / dt), 0.0);
-    const double hi = fmin(floor((tj + kGaborCut * sigma - t0) / dt), (double)(n_bins - 1));
-    if (!(lo <= hi)) return w;
-    // the bin of the window nearest to t_j
-    const double c = fmin(fmax(rint((tj - t0) / dt), lo), hi);
-    w.lo = (long long)lo;
-    w.hi = (long long)hi;
+    const GaborBins b = gabor_bins(tj, t0, dt, sigma, n_bins);
+    GaborWindow w{b.lo, b.hi, 0, b.nan ? tj : 0.0};
+    if (b.lo > b.hi) return w;
+    const double c = fmin(fmax(rint((tj - t0) / dt), (double)b.lo), (double)b.hi);
     w.c = (long long)c;
     w.delta = (t0 + c * dt) - tj;
     return w;
