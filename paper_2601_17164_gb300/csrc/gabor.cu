@@ -32,7 +32,8 @@
 // Emission time: a block of 16 warps per 32 frequencies scans |G(t_j, w)|^2 over the
 // analysis times in [t_a, t_b] for the centroid and the peak (vertex of the parabola
 // through ln|G|^2 at the maximum and its two neighbours); 122 -> 28 us at
-// the same size (one thread per frequency before).
+// the same size (one thread per frequency before, which is still the faster form for few
+// times or very many frequencies: launch_emission_time).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -248,23 +249,24 @@ __global__ void __cluster_dims__(1, 1, kHalves) __launch_bounds__(kGThreads)
 }
 
 constexpr int kEWarps = 16;
+constexpr int kEDirect = 128;   // threads of a block with one thread per frequency
 
-__global__ void __launch_bounds__(32 * kEWarps)
+// kWarps warps per 32 frequencies (kEWarps: a block; 1: every warp by itself)
+template <int kWarps>
+__global__ void __launch_bounds__(kWarps == 1 ? kEDirect : 32 * kWarps)
     emission_kernel(const double* __restrict__ g_re, const double* __restrict__ g_im, int64_t n_t, int64_t n_omega,
                     const double* __restrict__ times, double t_a, double t_b, double* centroid, double* peak) {
-    __shared__ double s_s0[kEWarps][32], s_s1[kEWarps][32], s_p[kEWarps][32];
-    __shared__ long long s_j[kEWarps][32], s_first[kEWarps], s_last[kEWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t m = (int64_t)blockIdx.x * 32 + lane;
+    const int lane = threadIdx.x & 31, warp = kWarps == 1 ? 0 : threadIdx.x >> 5;
+    const int64_t m = kWarps == 1 ? (int64_t)blockIdx.x * kEDirect + threadIdx.x : (int64_t)blockIdx.x * 32 + lane;
     const bool have = m < n_omega;
     auto P = [&](int64_t j) {
         const double r = g_re[j * n_omega + m], i = g_im[j * n_omega + m];
         return r * r + i * i;
     };
-    // warp q takes the times q, q + 16, ...
+    // warp q takes the times q, q + kWarps, ...
     double s0 = 0.0, s1 = 0.0, pmax = -1.0;
     int64_t jmax = -1, j_first = LLONG_MAX, j_last = -1;
-    for (int64_t j = warp; j < n_t; j += kEWarps) {
+    for (int64_t j = warp; j < n_t; j += kWarps) {
         const double t = times[j];
         if (!(t >= t_a && t <= t_b)) continue;
         if (j < j_first) j_first = j;
@@ -278,29 +280,34 @@ __global__ void __launch_bounds__(32 * kEWarps)
             jmax = j;
         }
     }
-    s_s0[warp][lane] = s0;
-    s_s1[warp][lane] = s1;
-    s_p[warp][lane] = pmax;
-    s_j[warp][lane] = jmax;
-    if (lane == 0) {
-        s_first[warp] = j_first;
-        s_last[warp] = j_last;
-    }
-    __syncthreads();
-    if (warp != 0 || !have) return;
-    for (int q = 1; q < kEWarps; ++q) {
-        s0 += s_s0[q][lane];
-        s1 += s_s1[q][lane];
-        const double p = s_p[q][lane];
-        const int64_t j = s_j[q][lane];
-        // the first of equal maxima
-        if (j >= 0 && (p > pmax || (p == pmax && j < jmax))) {
-            pmax = p;
-            jmax = j;
+    if constexpr (kWarps > 1) {
+        __shared__ double s_s0[kWarps][32], s_s1[kWarps][32], s_p[kWarps][32];
+        __shared__ long long s_j[kWarps][32], s_first[kWarps], s_last[kWarps];
+        s_s0[warp][lane] = s0;
+        s_s1[warp][lane] = s1;
+        s_p[warp][lane] = pmax;
+        s_j[warp][lane] = jmax;
+        if (lane == 0) {
+            s_first[warp] = j_first;
+            s_last[warp] = j_last;
         }
-        if (s_first[q] < j_first) j_first = s_first[q];
-        if (s_last[q] > j_last) j_last = s_last[q];
+        __syncthreads();
+        if (warp != 0) return;
+        for (int q = 1; q < kWarps; ++q) {
+            s0 += s_s0[q][lane];
+            s1 += s_s1[q][lane];
+            const double p = s_p[q][lane];
+            const int64_t j = s_j[q][lane];
+            // the first of equal maxima
+            if (j >= 0 && (p > pmax || (p == pmax && j < jmax))) {
+                pmax = p;
+                jmax = j;
+            }
+            if (s_first[q] < j_first) j_first = s_first[q];
+            if (s_last[q] > j_last) j_last = s_last[q];
+        }
     }
+    if (!have) return;
     double cen = nan(""), pk = nan("");
     if (jmax >= 0 && s0 > 0.0) {
         cen = s1 / s0;
@@ -344,8 +351,15 @@ cudaError_t launch_emission_time(const double* g_re, const double* g_im, int64_t
                                  const double* times, double t_a, double t_b, double* centroid, double* peak,
                                  cudaStream_t s) {
     if (n_omega == 0) return cudaSuccess;
-    emission_kernel<<<(unsigned)((n_omega + 31) / 32), 32 * kEWarps, 0, s>>>(g_re, g_im, n_t, n_omega, times, t_a,
-                                                                             t_b, centroid, peak);
+    // One thread per frequency where its few times, or its many frequencies, leave 16 warps
+    // nothing to share (152 SMs; its time over that of 16 warps): 3 times 0.92, 10 times 1.2 up
+    // to 5000 frequencies; 20000: 0.76 at 20 times, 0.99 at 50; 1e5: 0.90 at 100, 1.15 at 400.
+    if (n_t < std::max<int64_t>(6, (n_omega - 3000) / 400))
+        emission_kernel<1><<<(unsigned)((n_omega + kEDirect - 1) / kEDirect), kEDirect, 0, s>>>(
+            g_re, g_im, n_t, n_omega, times, t_a, t_b, centroid, peak);
+    else
+        emission_kernel<kEWarps><<<(unsigned)((n_omega + 31) / 32), 32 * kEWarps, 0, s>>>(
+            g_re, g_im, n_t, n_omega, times, t_a, t_b, centroid, peak);
     return cudaGetLastError();
 }
 
