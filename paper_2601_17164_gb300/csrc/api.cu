@@ -766,14 +766,15 @@ static sfhk_status run_traj(const sfhk_field* field, const sfhk_target* target, 
         a.esc_ratio = pp->esc_ratio;
     }
     // FP64 endpoints, and the FP64 planar dipole into atomic bins: the warp-specialised
-    // kernels, up to the length at which the one-thread-per-trajectory kernel is faster; a
-    // caller's own launch shape (block, chunk_steps) asks for that one
+    // kernels, up to the length at which the one-thread-per-trajectory kernel is faster (and
+    // in dipoles up to the d_t that keeps |det Z|^2 in range); a caller's own launch shape
+    // (block, chunk_steps) asks for that one
     const bool warps64 = pp->precision == 0 && pp->block == 0 && pp->chunk_steps == 0;
     const int pot = target->t.pot;
     cudaError_t launched;
     if (warps64 && mode == 0 && n <= endpoints_limit(pot, a.redo_lists))
         launched = launch_endpoints(field->f, target->t, a, s);
-    else if (warps64 && a.planar && !det && n <= fp64_limit(pot, a.redo_lists))
+    else if (warps64 && a.planar && !det && pp->d_t <= kWarpsDt && n <= fp64_limit(pot, a.redo_lists))
         launched = launch_fp64(field->f, target->t, a, s);
     else launched = launch_traj(field->f, target->t, pp->precision, a, s);
     st = check_cuda(launched, "trajectory launch");

@@ -414,7 +414,7 @@ __device__ void quad_columns(const FieldDev& f, const TrajArgs& a, const QCommon
             in_q.release(di);
             const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, odd);
             turned = 0;
-            if (step) follow_branch8(Dp, D, sgn, turned);
+            if (step) follow_branch<double>(Dp, D, sgn, turned);
         }
     }
     out.drain();
@@ -568,7 +568,7 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
         if constexpr (FB) {
             // the step n -> n + 1: det Z of the advanced columns
             const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, l & 1);
-            if (alive && n >= c.n0 && n < c.n_last) follow_branch8(Dp, D, sgn, flags);
+            if (alive && n >= c.n0 && n < c.n_last) follow_branch<double>(Dp, D, sgn, flags);
         } else {
             if (c.have && n >= c.n0 && n < c.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, f.k64.h6);
         }

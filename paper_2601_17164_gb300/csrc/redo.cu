@@ -408,7 +408,7 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
                 T.bq = fma(oa, yb, fma(ob, pb, yb));
                 T.bp = fma(oc, yb, fma(od, pb, pb));
                 const Cx2<double> D = T.detc(1.0, -2.0 * rg, 2.0 * a.qg64);
-                follow_branch8(Dp, D, sgn, flags);
+                follow_branch<double>(Dp, D, sgn, flags);
                 ++all_steps;
                 if (n >= c.k_cnt) ++steps;
             }

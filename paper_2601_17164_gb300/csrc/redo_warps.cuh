@@ -1,7 +1,6 @@
 // Pieces shared by the warp-specialised FP64 kernels (redo.cu, quad.cu): the hand-off
 // rings between the warps of a block, the view of a planar state that the
-// recombination terms take, the root and branch of det Z, and where a block's groups
-// come from.
+// recombination terms take, the root of det Z, and where a block's groups come from.
 #pragma once
 
 #include "traj_block.cuh"
@@ -19,28 +18,14 @@ struct PView {
     __device__ PView(double q0, double q2, double p0, double p2, double s) : q{q0, 0.0, q2}, p{p0, 0.0, p2}, S{s} {}
 };
 
-// The principal root of D = det Z, m2 = |D|^2.  |D| is sqrt(m2) (an eighth of hypot's FP64
-// instructions) while m2 is a normal number that keeps its digits; a d_t above 1.3e154 lets
-// |D| grow past that, where c_sqrt's hypot is in range.
+// The principal root of D = det Z, m2 = |D|^2, with |D| = sqrt(m2): an eighth of hypot's
+// FP64 instructions.  Calls with d_t up to kWarpsDt come here, so |D| of a trajectory that
+// stays is at most that and m2 is in range (as are the products of 8 det Z that follow the
+// branch).
 __device__ __forceinline__ cd root_det(cd D, double m2) {
-    const int e = __double2hiint(m2);
-    if (e < 0x03f00000 || e >= 0x7ff00000) return c_sqrt(D);
     const double r = sqrt(m2);
     const double q = sqrt(0.5 * (r + fabs(D.re))), o = positive(q) ? D.im / (2.0 * q) : 0.0;
     return D.re >= 0.0 ? mk(q, o) : mk(fabs(o), copysign(q, D.im));
-}
-// follow_branch on 8 det Z: its products reach FP64's range at an eighth of the |det Z| at
-// which those of det Z do, so values of 2^496 or more are scaled back (exactly) first
-__device__ __forceinline__ void follow_branch8(Cx2<double>& Dp, Cx2<double> D, double& sgn, unsigned& flags) {
-    const unsigned e = max(max((unsigned)__double2hiint(Dp.re) << 1, (unsigned)__double2hiint(Dp.im) << 1),
-                           max((unsigned)__double2hiint(D.re) << 1, (unsigned)__double2hiint(D.im) << 1));
-    if (e < 0x5ef00000u << 1) {
-        follow_branch<double>(Dp, D, sgn, flags);
-        return;
-    }
-    Cx2<double> P{0.125 * Dp.re, 0.125 * Dp.im};
-    follow_branch<double>(P, Cx2<double>{0.125 * D.re, 0.125 * D.im}, sgn, flags);
-    Dp = D;
 }
 
 // Hand-offs of N slots between consecutive roles on named barriers (0 is left to

@@ -201,6 +201,9 @@ inline size_t redo_scratch_words(int64_t n, int64_t quad_limit) {
     return 3 * (size_t)kRedoLists + 2 * (size_t)redo_groups(n, quad_limit);
 }
 cudaError_t launch_quad(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
+// largest d_t for which the warp-specialised kernels form |det Z|^2 and 8 det Z (MIXED calls
+// have 1e36 at most): beyond, the one-thread kernel's hypot is in range
+constexpr double kWarpsDt = 1e150;
 // the FP64 planar dipole of births [0, n) by the same kernels, without escalation list or
 // scratch, up to the longest call they take
 int64_t fp64_limit(int pot, int sms);
