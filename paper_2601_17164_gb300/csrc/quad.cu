@@ -66,7 +66,7 @@ struct QShared {
     double hess[4 * 3 * kT];   // stage Hessians (a, b, c), matrix warp only
     double phase[16][2];       // cos and -sin of Ip t at bin k in row k & 15 (float bins)
     int alive[kT];             // written by the bins warp, read late by the warps ahead
-    long long last;            // the group's last grid point (GroupEnd)
+    long long last;            // the group's last grid point when it ends early, else -1 (GroupEnd)
 };
 
 struct QCommon {
@@ -165,55 +165,57 @@ __device__ void quad_dynamics(const FieldDev& f, const TargetDev& tg, const Traj
     };
     int rem = (int)(cm.n_first % cm.n_out);
     int64_t k_bin = (cm.n_first + cm.n_out - 1) / cm.n_out;
-    GroupEnd end(sm.last);
-    for (int64_t n = cm.n_first; n <= end.last; ++n) {
-        const int d = out.acquire();
-        const bool live = alive[t];
-        end.decide(n, live);
-        // float bins: e^{-i Ip t} of the bin at this grid point (this warp has the FP64
-        // instructions to spare; the hand-offs keep the bins warp less than 16 grid points
-        // behind, so a row is read before its next use even with a bin at every point)
-        if (FB && rem == 0) {
-            if (threadIdx.x % 32 == 0) {
-                double sn, cs;
-                sincos(bin_phase(f, tg, n), &sn, &cs);
-                sm.phase[k_bin & 15][0] = cs;
-                sm.phase[k_bin & 15][1] = -sn;
+    for (int64_t n = cm.n_first; n <= cm.n_last;) {
+        int left = GroupEnd::stretch(n, cm.n_last);
+        GroupEnd::decide(sm.last, n + left - 1, alive[t]);
+        for (; left > 0; --left, ++n) {
+            const int d = out.acquire();
+            // float bins: e^{-i Ip t} of the bin at this grid point (this warp has the FP64
+            // instructions to spare; the hand-offs keep the bins warp less than 16 grid points
+            // behind, so a row is read before its next use even with a bin at every point)
+            if (FB && rem == 0) {
+                if (threadIdx.x % 32 == 0) {
+                    double sn, cs;
+                    sincos(bin_phase(f, tg, n), &sn, &cs);
+                    sm.phase[k_bin & 15][0] = cs;
+                    sm.phase[k_bin & 15][1] = -sn;
+                }
+                ++k_bin;
             }
-            ++k_bin;
+            rem = (rem + 1 == cm.n_out) ? 0 : rem + 1;
+            double* const o = sm.s01[d] + t;
+            const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
+            const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
+            double g;
+            const double qa = pair ? fma(hk.hh, p1, q1) : q1;                       // Q1, Q2
+            const double ka = force(qa, pair ? e1 : e0, o + pair * kStage, g);      // F1, F2
+            const double pn = fma(hk.hh, ka, p1);                                   // P2, P3
+            const double qb = fma(pair ? hk.h : hk.hh, pn, q1);                     // Q3, Q4
+            const double kb = force(qb, pair ? e2 : e1, o + (2 + pair) * kStage, g);   // F3, F4
+            const double p4 = fma(hk.h, kb, p1);                                    // (P4 in the first pair)
+            // stage momenta: P2 and P3, P1 and P4
+            o[(1 + pair) * kStage + (4 + c) * kT] = pn;
+            const double p4_o = xor_lane(p4, 2 * kT);
+            o[(pair ? 3 * kStage : 0) + (4 + c) * kT] = pair ? p4_o : p1;
+            out.publish(d);
+            // the RK4 combination, q_c in the first pair and p_c in the second; the last term of
+            // p_x' is -g x' unrounded (so nvcc contracts it in the other FP64 kernels: found by
+            // comparing chaotic trajectories)
+            const double pn_o = xor_lane(pn, 2 * kT), ka_o = xor_lane(ka, 2 * kT), kb_o = xor_lane(kb, 2 * kT);
+            const double s3 = fma(2.0, (pair ? ka : pn) + (pair ? kb_o : pn_o), pair ? ka_o : p1);
+            const bool px = pair && c == 0;
+            const double s = fma(px ? -g : 1.0, px ? qb : (pair ? kb : p4), s3);
+            const double nb = fma(hk.h6, s, pair ? p1 : q1);
+            const double no = xor_lane(nb, 2 * kT);
+            if (step) {
+                q1 = pair ? no : nb;
+                p1 = pair ? nb : no;
+            }
+            e0 = f0;
+            e1 = f1;
+            e2 = f2;
         }
-        rem = (rem + 1 == cm.n_out) ? 0 : rem + 1;
-        double* const o = sm.s01[d] + t;
-        const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
-        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && live;
-        double g;
-        const double qa = pair ? fma(hk.hh, p1, q1) : q1;                       // Q1, Q2
-        const double ka = force(qa, pair ? e1 : e0, o + pair * kStage, g);      // F1, F2
-        const double pn = fma(hk.hh, ka, p1);                                   // P2, P3
-        const double qb = fma(pair ? hk.h : hk.hh, pn, q1);                     // Q3, Q4
-        const double kb = force(qb, pair ? e2 : e1, o + (2 + pair) * kStage, g);   // F3, F4
-        const double p4 = fma(hk.h, kb, p1);                                    // (P4 in the first pair)
-        // stage momenta: P2 and P3, P1 and P4
-        o[(1 + pair) * kStage + (4 + c) * kT] = pn;
-        const double p4_o = xor_lane(p4, 2 * kT);
-        o[(pair ? 3 * kStage : 0) + (4 + c) * kT] = pair ? p4_o : p1;
-        out.publish(d);
-        // the RK4 combination, q_c in the first pair and p_c in the second; the last term of
-        // p_x' is -g x' unrounded (so nvcc contracts it in the other FP64 kernels: found by
-        // comparing chaotic trajectories)
-        const double pn_o = xor_lane(pn, 2 * kT), ka_o = xor_lane(ka, 2 * kT), kb_o = xor_lane(kb, 2 * kT);
-        const double s3 = fma(2.0, (pair ? ka : pn) + (pair ? kb_o : pn_o), pair ? ka_o : p1);
-        const bool px = pair && c == 0;
-        const double s = fma(px ? -g : 1.0, px ? qb : (pair ? kb : p4), s3);
-        const double nb = fma(hk.h6, s, pair ? p1 : q1);
-        const double no = xor_lane(nb, 2 * kT);
-        if (step) {
-            q1 = pair ? no : nb;
-            p1 = pair ? nb : no;
-        }
-        e0 = f0;
-        e1 = f1;
-        e2 = f2;
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -275,68 +277,70 @@ __device__ void quad_matrix(const FieldDev& f, const TargetDev& tg, const QCommo
     Consumer<2> in_q(kHand0);
     Producer<2> out(kHand1);
     const double h = hk.h, c2 = hk.c2, c4 = hk.c4, c3 = hk.c3, c1 = hk.h6;
-    GroupEnd end(sm.last);
-    for (int64_t n = cm.n_first; n <= end.last; ++n) {
-        const double e_next = e_at(2 * n + 2 + e_off);
-        const int di = in_q.wait();
-        end.follow();
-        const double* const in = sm.s01[di] + t;
-        // stage l: Hessian data and the action integrand
-        const double* const st = in + l * kStage;
-        const double x = st[0], z = st[kT], g = st[2 * kT], px = st[4 * kT], pz = st[5 * kT];
-        double hs, V;
-        if constexpr (POT == POT_SOFTCORE) {
-            hs = -3.0 * g * st[6 * kT];
-            V = -st[3 * kT];
-        } else if constexpr (POT == POT_TONGLIN) {
-            const double ir = st[3 * kT], Y = st[6 * kT], Y1 = st[7 * kT];
-            const double r = fma(x, x, z * z) * ir;
-            hs = tonglin_h(pc, r, ir, Y, Y1, st[8 * kT], st[9 * kT], st[10 * kT]);
-            V = -Y * ir;
-        } else if constexpr (POT == POT_HARMONIC) {
-            hs = 0.0;
-            V = 0.5 * pc.a2 * fma(x, x, z * z);
-        } else {
-            hs = 0.0;
-            V = 0.0;
-        }
-        const double hx = hs * x;
-        double* const H = sm.hess + t;
-        H[(3 * l) * kT] = fma(hx, x, g);
-        H[(3 * l + 1) * kT] = hx * z;
-        H[(3 * l + 2) * kT] = fma(hs * z, z, g);
-        const double kS = TrajP<double, POT>::action_term(px, pz, z, e_cur, V);
-        const double g0 = in[2 * kT], g1 = in[kStage + 2 * kT], g2 = in[2 * kStage + 2 * kT],
-                     g3 = in[3 * kStage + 2 * kT];
-        const double state_l = in[(l < 2 ? l : l + 2) * kT];   // q_x', q_z, p_x', p_z at n
-        in_q.release(di);
-        __syncwarp();
-        const int dq = out.acquire();
-        double* const o = sm.s12[dq] + t;
-        // entry (ei, ej) from row ei of H3, H4 and column ej of H1, H2
-        auto He = [&](int s, int i, int j) { return H[(3 * s + i + j) * kT]; };
-        const double h0e = He(0, ei, ej), h1e = He(1, ei, ej), h2e = He(2, ei, ej), h3e = He(3, ei, ej);
-        const double p31 = fma(He(2, ei, 0), He(0, 0, ej), He(2, ei, 1) * He(0, 1, ej));
-        const double p42 = fma(He(3, ei, 0), He(1, 0, ej), He(3, ei, 1) * He(1, 1, ej));
-        __syncwarp();   // the Hessians are read before the next grid point writes them
-        const double s23 = h1e + h2e;
-        o[l * kT] = fma(c4, p31, -c2 * (s23 + h0e));
-        o[(4 + l) * kT] = fma(-c3, s23, ei == ej ? h : 0.0);
-        o[(8 + l) * kT] = fma(c3, p31 + p42, -c1 * (fma(2.0, s23, h0e) + h3e));
-        o[(12 + l) * kT] = fma(c4, p42, -c2 * (s23 + h3e));
-        if constexpr (FB) {
-            o[(kM + l) * kT] = l == 0 ? g0 : (l == 1 ? g1 : (l == 2 ? g2 : g3));
-        } else {
-            const double2 r = out_of_plane(hk, g0, g1, g2, g3, odd);
-            if (l < 2) {
-                o[(kM + 2 * l) * kT] = r.x;
-                o[(kM + 2 * l + 1) * kT] = r.y;
+    for (int64_t n = cm.n_first; n <= cm.n_last;) {
+        int left = GroupEnd::stretch(n, cm.n_last);
+        for (; left > 0; --left, ++n) {
+            const double e_next = e_at(2 * n + 2 + e_off);
+            const int di = in_q.wait();
+            const double* const in = sm.s01[di] + t;
+            // stage l: Hessian data and the action integrand
+            const double* const st = in + l * kStage;
+            const double x = st[0], z = st[kT], g = st[2 * kT], px = st[4 * kT], pz = st[5 * kT];
+            double hs, V;
+            if constexpr (POT == POT_SOFTCORE) {
+                hs = -3.0 * g * st[6 * kT];
+                V = -st[3 * kT];
+            } else if constexpr (POT == POT_TONGLIN) {
+                const double ir = st[3 * kT], Y = st[6 * kT], Y1 = st[7 * kT];
+                const double r = fma(x, x, z * z) * ir;
+                hs = tonglin_h(pc, r, ir, Y, Y1, st[8 * kT], st[9 * kT], st[10 * kT]);
+                V = -Y * ir;
+            } else if constexpr (POT == POT_HARMONIC) {
+                hs = 0.0;
+                V = 0.5 * pc.a2 * fma(x, x, z * z);
+            } else {
+                hs = 0.0;
+                V = 0.0;
             }
+            const double hx = hs * x;
+            double* const H = sm.hess + t;
+            H[(3 * l) * kT] = fma(hx, x, g);
+            H[(3 * l + 1) * kT] = hx * z;
+            H[(3 * l + 2) * kT] = fma(hs * z, z, g);
+            const double kS = TrajP<double, POT>::action_term(px, pz, z, e_cur, V);
+            const double g0 = in[2 * kT], g1 = in[kStage + 2 * kT], g2 = in[2 * kStage + 2 * kT],
+                         g3 = in[3 * kStage + 2 * kT];
+            const double state_l = in[(l < 2 ? l : l + 2) * kT];   // q_x', q_z, p_x', p_z at n
+            in_q.release(di);
+            __syncwarp();
+            const int dq = out.acquire();
+            double* const o = sm.s12[dq] + t;
+            // entry (ei, ej) from row ei of H3, H4 and column ej of H1, H2
+            auto He = [&](int s, int i, int j) { return H[(3 * s + i + j) * kT]; };
+            const double h0e = He(0, ei, ej), h1e = He(1, ei, ej), h2e = He(2, ei, ej), h3e = He(3, ei, ej);
+            const double p31 = fma(He(2, ei, 0), He(0, 0, ej), He(2, ei, 1) * He(0, 1, ej));
+            const double p42 = fma(He(3, ei, 0), He(1, 0, ej), He(3, ei, 1) * He(1, 1, ej));
+            __syncwarp();   // the Hessians are read before the next grid point writes them
+            const double s23 = h1e + h2e;
+            o[l * kT] = fma(c4, p31, -c2 * (s23 + h0e));
+            o[(4 + l) * kT] = fma(-c3, s23, ei == ej ? h : 0.0);
+            o[(8 + l) * kT] = fma(c3, p31 + p42, -c1 * (fma(2.0, s23, h0e) + h3e));
+            o[(12 + l) * kT] = fma(c4, p42, -c2 * (s23 + h3e));
+            if constexpr (FB) {
+                o[(kM + l) * kT] = l == 0 ? g0 : (l == 1 ? g1 : (l == 2 ? g2 : g3));
+            } else {
+                const double2 r = out_of_plane(hk, g0, g1, g2, g3, odd);
+                if (l < 2) {
+                    o[(kM + 2 * l) * kT] = r.x;
+                    o[(kM + 2 * l + 1) * kT] = r.y;
+                }
+            }
+            o[(kState + l) * kT] = state_l;
+            o[(kAct + l) * kT] = kS;
+            out.publish(dq);
+            e_cur = e_next;
         }
-        o[(kState + l) * kT] = state_l;
-        o[(kAct + l) * kT] = kS;
-        out.publish(dq);
-        e_cur = e_next;
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -359,63 +363,65 @@ __device__ void quad_columns(const FieldDev& f, const TrajArgs& a, const QCommon
     const volatile int* alive = sm.alive;
     Consumer<2> in_q(kHand1);
     Producer<3> out(kHand2);
-    GroupEnd end(sm.last);
-    for (int64_t n = cm.n_first; n <= end.last; ++n) {
-        const int di = in_q.wait();
-        end.follow();
-        const double* const in = sm.s12[di] + t;
-        int dq = 0;
-        if constexpr (!FB) {
-            dq = out.acquire();
-            double* const o = sm.s23[dq] + t;
-            // 8 det Z at grid point n: re, im, the branch's sign (doubled after a turn)
-            if (l < 3) o[(kDetD + l) * kT] = l == 0 ? Dp.re : (l == 1 ? Dp.im : (turned ? 2.0 * sgn : sgn));
-            o[l * kT] = in[(kState + l) * kT];
-            o[(4 + l) * kT] = in[(kAct + l) * kT];
-            out.publish(dq);
+    for (int64_t n = cm.n_first; n <= cm.n_last;) {
+        int left = GroupEnd::stretch(n, cm.n_last);
+        for (; left > 0; --left, ++n) {
+            const int di = in_q.wait();
+            const double* const in = sm.s12[di] + t;
+            int dq = 0;
+            if constexpr (!FB) {
+                dq = out.acquire();
+                double* const o = sm.s23[dq] + t;
+                // 8 det Z at grid point n: re, im, the branch's sign (doubled after a turn)
+                if (l < 3) o[(kDetD + l) * kT] = l == 0 ? Dp.re : (l == 1 ? Dp.im : (turned ? 2.0 * sgn : sgn));
+                o[l * kT] = in[(kState + l) * kT];
+                o[(4 + l) * kT] = in[(kAct + l) * kT];
+                out.publish(dq);
+            }
+            const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
+            const double wp = xor_lane(w, kT);   // the other entry of this out-of-plane column
+            double m0, m1;
+            if constexpr (FB) {
+                const double2 r = out_of_plane(hk, in[kM * kT], in[(kM + 1) * kT], in[(kM + 2) * kT], in[(kM + 3) * kT], odd);
+                m0 = r.x;
+                m1 = r.y;
+            } else {
+                m0 = in[(kM + 2 * odd) * kT];
+                m1 = in[(kM + 2 * odd + 1) * kT];
+            }
+            if (step) {
+                const double x0 = X0, x1 = X1, y0 = Y0, y1 = Y1;
+                X0 = fma(in[0], x0, fma(in[kT], x1, fma(in[4 * kT], y0, fma(in[5 * kT], y1, x0))));
+                X1 = fma(in[2 * kT], x0, fma(in[3 * kT], x1, fma(in[5 * kT], y0, fma(in[7 * kT], y1, x1))));
+                Y0 = fma(in[8 * kT], x0, fma(in[9 * kT], x1, fma(in[12 * kT], y0, fma(in[13 * kT], y1, y0))));
+                Y1 = fma(in[10 * kT], x0, fma(in[11 * kT], x1, fma(in[14 * kT], y0, fma(in[15 * kT], y1, y1))));
+                const double q = odd ? wp : w, p = odd ? w : wp;
+                w = fma(m0, q, fma(m1, p, w));
+            }
+            if constexpr (FB) {
+                const double state_l = in[(kState + l) * kT], s_n = S;
+                if (cm.have && n >= cm.n0 && n < cm.n_last)
+                    S += TrajP<double, POT>::action_sum(in[kAct * kT], in[(kAct + 1) * kT], in[(kAct + 2) * kT],
+                                                        in[(kAct + 3) * kT], hk.h6);
+                in_q.release(di);
+                dq = out.acquire();
+                double* const o = sm.s23[dq] + t;
+                o[l * kT] = state_l;
+                if (l == 0) o[4 * kT] = s_n;
+                o[(kDetF + 4 * l) * kT] = X0;
+                o[(kDetF + 4 * l + 1) * kT] = X1;
+                o[(kDetF + 4 * l + 2) * kT] = Y0;
+                o[(kDetF + 4 * l + 3) * kT] = Y1;
+                o[(kDetF + 16 + l) * kT] = w;
+                out.publish(dq);
+            } else {
+                in_q.release(di);
+                const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, odd);
+                turned = 0;
+                if (step) follow_branch<double>(Dp, D, sgn, turned);
+            }
         }
-        const bool step = cm.have && n >= cm.n0 && n < cm.n_last && alive[t];
-        const double wp = xor_lane(w, kT);   // the other entry of this out-of-plane column
-        double m0, m1;
-        if constexpr (FB) {
-            const double2 r = out_of_plane(hk, in[kM * kT], in[(kM + 1) * kT], in[(kM + 2) * kT], in[(kM + 3) * kT], odd);
-            m0 = r.x;
-            m1 = r.y;
-        } else {
-            m0 = in[(kM + 2 * odd) * kT];
-            m1 = in[(kM + 2 * odd + 1) * kT];
-        }
-        if (step) {
-            const double x0 = X0, x1 = X1, y0 = Y0, y1 = Y1;
-            X0 = fma(in[0], x0, fma(in[kT], x1, fma(in[4 * kT], y0, fma(in[5 * kT], y1, x0))));
-            X1 = fma(in[2 * kT], x0, fma(in[3 * kT], x1, fma(in[5 * kT], y0, fma(in[7 * kT], y1, x1))));
-            Y0 = fma(in[8 * kT], x0, fma(in[9 * kT], x1, fma(in[12 * kT], y0, fma(in[13 * kT], y1, y0))));
-            Y1 = fma(in[10 * kT], x0, fma(in[11 * kT], x1, fma(in[14 * kT], y0, fma(in[15 * kT], y1, y1))));
-            const double q = odd ? wp : w, p = odd ? w : wp;
-            w = fma(m0, q, fma(m1, p, w));
-        }
-        if constexpr (FB) {
-            const double state_l = in[(kState + l) * kT], s_n = S;
-            if (cm.have && n >= cm.n0 && n < cm.n_last)
-                S += TrajP<double, POT>::action_sum(in[kAct * kT], in[(kAct + 1) * kT], in[(kAct + 2) * kT],
-                                                    in[(kAct + 3) * kT], hk.h6);
-            in_q.release(di);
-            dq = out.acquire();
-            double* const o = sm.s23[dq] + t;
-            o[l * kT] = state_l;
-            if (l == 0) o[4 * kT] = s_n;
-            o[(kDetF + 4 * l) * kT] = X0;
-            o[(kDetF + 4 * l + 1) * kT] = X1;
-            o[(kDetF + 4 * l + 2) * kT] = Y0;
-            o[(kDetF + 4 * l + 3) * kT] = Y1;
-            o[(kDetF + 16 + l) * kT] = w;
-            out.publish(dq);
-        } else {
-            in_q.release(di);
-            const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, odd);
-            turned = 0;
-            if (step) follow_branch<double>(Dp, D, sgn, turned);
-        }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -443,139 +449,141 @@ __device__ void quad_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms
     int64_t k_bin = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
     Consumer<3> in_q(kHand2);
-    GroupEnd end(sm.last);
-    for (int64_t n = c.n_first; n <= end.last; ++n) {
-        const int di = in_q.wait();
-        end.follow();
-        const double* const in = sm.s23[di] + t;
-        const double q0 = in[0], q2 = in[kT], p0 = in[2 * kT], p2 = in[3 * kT];
-        double k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0;
-        double X0 = 0.0, X1 = 0.0, Y0 = 0.0, Y1 = 0.0, w = 0.0;
-        if constexpr (FB) {
-            S = in[4 * kT];
-            X0 = in[(kDetF + 4 * l) * kT];
-            X1 = in[(kDetF + 4 * l + 1) * kT];
-            Y0 = in[(kDetF + 4 * l + 2) * kT];
-            Y1 = in[(kDetF + 4 * l + 3) * kT];
-            w = in[(kDetF + 16 + l) * kT];
-        } else {
-            k1 = in[4 * kT];
-            k2 = in[5 * kT];
-            k3 = in[6 * kT];
-            k4 = in[7 * kT];
-            Dp = Cx2<double>{in[kDetD * kT], in[(kDetD + 1) * kT]};
-            sgn = in[(kDetD + 2) * kT];
-        }
-        in_q.release(di);
-        const bool on_bin = rem == 0;
-        if (!FB && alive && (__double2hiint(sgn) & 0x7fffffff) == 0x40000000) flags |= 4u;   // |sgn| = 2
-        // partial waves (Sec. III.A-B), as in redo.cu
-        if (pw && alive && n >= c.n0) {
-            const double qx = q0, qy = 0.0, qzz = q2;
-            const bool inside = qx * qx + qy * qy + qzz * qzz < pw_r2;
-            if (inside && !pw_in) {
-                const double px = p0, py = 0.0, pz = p2;
-                const double lx = qy * pz - qzz * py, ly = qzz * px - qx * pz, lz = qx * py - qy * px;
-                const double L2 = lx * lx + ly * ly + lz * lz;
-                pw_cls = L2 < 0.25 ? 0 : (L2 < 2.25 ? 1 : (L2 < 6.25 ? 2 : 3));
+    for (int64_t n = c.n_first; n <= c.n_last;) {
+        int left = GroupEnd::stretch(n, c.n_last);
+        for (; left > 0; --left, ++n) {
+            const int di = in_q.wait();
+            const double* const in = sm.s23[di] + t;
+            const double q0 = in[0], q2 = in[kT], p0 = in[2 * kT], p2 = in[3 * kT];
+            double k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0;
+            double X0 = 0.0, X1 = 0.0, Y0 = 0.0, Y1 = 0.0, w = 0.0;
+            if constexpr (FB) {
+                S = in[4 * kT];
+                X0 = in[(kDetF + 4 * l) * kT];
+                X1 = in[(kDetF + 4 * l + 1) * kT];
+                Y0 = in[(kDetF + 4 * l + 2) * kT];
+                Y1 = in[(kDetF + 4 * l + 3) * kT];
+                w = in[(kDetF + 16 + l) * kT];
+            } else {
+                k1 = in[4 * kT];
+                k2 = in[5 * kT];
+                k3 = in[6 * kT];
+                k4 = in[7 * kT];
+                Dp = Cx2<double>{in[kDetD * kT], in[(kDetD + 1) * kT]};
+                sgn = in[(kDetD + 2) * kT];
             }
-            pw_in = inside;
-        }
-        const bool pw_ok = !pw || (pw_cls >= 0 && ((a.pw_mask >> pw_cls) & 1));
-        if (on_bin) {
-            bool valid = false;
-            Cx<double> C{0.0, 0.0};
-            if (alive && n >= c.n0) {
-                const cd D = 0.125 * cd{Dp.re, Dp.im};
-                const double fs = q0 + q2 + p0 + p2;
-                const bool ok = isfinite(fs) && isfinite(S);
-                const double m2 = D.re * D.re + D.im * D.im;
-                if (!ok || !(m2 <= a.d_t * a.d_t)) {
-                    alive = false;
-                    flags |= 1u;
-                    if (!ok || !isfinite(m2)) flags |= 2u;
-                } else if (n >= c.k_cnt && pw_ok) {
-                    cd Cz = root_det(D, m2);
-                    if (sgn < 0.0) Cz = -Cz;
-                    C = Cx<double>{Cz.re, Cz.im};
-                    valid = true;
+            in_q.release(di);
+            const bool on_bin = rem == 0;
+            if (!FB && alive && (__double2hiint(sgn) & 0x7fffffff) == 0x40000000) flags |= 4u;   // |sgn| = 2
+            // partial waves (Sec. III.A-B), as in redo.cu
+            if (pw && alive && n >= c.n0) {
+                const double qx = q0, qy = 0.0, qzz = q2;
+                const bool inside = qx * qx + qy * qy + qzz * qzz < pw_r2;
+                if (inside && !pw_in) {
+                    const double px = p0, py = 0.0, pz = p2;
+                    const double lx = qy * pz - qzz * py, ly = qzz * px - qx * pz, lz = qx * py - qy * px;
+                    const double L2 = lx * lx + ly * ly + lz * lz;
+                    pw_cls = L2 < 0.25 ? 0 : (L2 < 2.25 ? 1 : (L2 < 6.25 ? 2 : 3));
                 }
+                pw_in = inside;
             }
-            if (__any_sync(0xffffffffu, valid)) {
-                double cl = 0.0, cv = 0.0;
-                if constexpr (FB) {
-                    if (valid && l == 0) {
-                        const FloatState fsn(q0, 0.0, q2, p0, 0.0, p2, S);
-                        float fl, fv;
-                        contribution<float>(fsn, gt, gamf, Cx<float>{(float)C.re, (float)C.im},
-                                            Cx<float>{(float)amp.re, (float)amp.im},
-                                            Cx<float>{(float)sm.phase[k_bin & 15][0], (float)sm.phase[k_bin & 15][1]}, fl, fv);
-                        cl = (double)fl;
-                        cv = (double)fv;
+            const bool pw_ok = !pw || (pw_cls >= 0 && ((a.pw_mask >> pw_cls) & 1));
+            if (on_bin) {
+                bool valid = false;
+                Cx<double> C{0.0, 0.0};
+                if (alive && n >= c.n0) {
+                    const cd D = 0.125 * cd{Dp.re, Dp.im};
+                    const double fs = q0 + q2 + p0 + p2;
+                    const bool ok = isfinite(fs) && isfinite(S);
+                    const double m2 = D.re * D.re + D.im * D.im;
+                    if (!ok || !(m2 <= a.d_t * a.d_t)) {
+                        alive = false;
+                        flags |= 1u;
+                        if (!ok || !isfinite(m2)) flags |= 2u;
+                    } else if (n >= c.k_cnt && pw_ok) {
+                        cd Cz = root_det(D, m2);
+                        if (sgn < 0.0) Cz = -Cz;
+                        C = Cx<double>{Cz.re, Cz.im};
+                        valid = true;
                     }
-                } else {
-                    // e^{-i Ip t} in even lanes and e^{i S} in odd lanes
-                    double sn, cs;
-                    sincos((l & 1) ? S : bin_phase(f, tg, n), &sn, &cs);
-                    const double sn_o = xor_lane(sn, kT), cs_o = xor_lane(cs, kT);   // lane 0: e^{i S}
-                    // the GTO terms in four parts
-                    const PView v(q0, q2, p0, p2, S);
-                    double pp, qq, pq;
-                    recomb_invariants<double>(v, pp, qq, pq);
-                    const float ppf = (float)pp, qqf = (float)qq;
-                    float most = -INFINITY;
-                    for (int j = l; j < gt.n; j += 4) most = fmaxf(most, gto_size(gt, ppf, qqf, j));
-                    most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, kT));
-                    most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, 2 * kT));
-                    GtoSums<double> g{};
-                    for (int j = l; j < gt.n; j += 4)
-                        if (valid && !(gto_size(gt, ppf, qqf, j) < most - kGtoNothing))
-                            gto_terms<double>(gt, pp, qq, pq, j, j + 1, g);
-                    auto fold = [](double& x) {
-                        x += xor_lane(x, kT);
-                        x += xor_lane(x, 2 * kT);
-                    };
+                }
+                if (__any_sync(0xffffffffu, valid)) {
+                    double cl = 0.0, cv = 0.0;
+                    if constexpr (FB) {
+                        if (valid && l == 0) {
+                            const FloatState fsn(q0, 0.0, q2, p0, 0.0, p2, S);
+                            float fl, fv;
+                            contribution<float>(fsn, gt, gamf, Cx<float>{(float)C.re, (float)C.im},
+                                                Cx<float>{(float)amp.re, (float)amp.im},
+                                                Cx<float>{(float)sm.phase[k_bin & 15][0], (float)sm.phase[k_bin & 15][1]}, fl, fv);
+                            cl = (double)fl;
+                            cv = (double)fv;
+                        }
+                    } else {
+                        // e^{-i Ip t} in even lanes and e^{i S} in odd lanes
+                        double sn, cs;
+                        sincos((l & 1) ? S : bin_phase(f, tg, n), &sn, &cs);
+                        const double sn_o = xor_lane(sn, kT), cs_o = xor_lane(cs, kT);   // lane 0: e^{i S}
+                        // the GTO terms in four parts
+                        const PView v(q0, q2, p0, p2, S);
+                        double pp, qq, pq;
+                        recomb_invariants<double>(v, pp, qq, pq);
+                        const float ppf = (float)pp, qqf = (float)qq;
+                        float most = -INFINITY;
+                        for (int j = l; j < gt.n; j += 4) most = fmaxf(most, gto_size(gt, ppf, qqf, j));
+                        most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, kT));
+                        most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, 2 * kT));
+                        GtoSums<double> g{};
+                        for (int j = l; j < gt.n; j += 4)
+                            if (valid && !(gto_size(gt, ppf, qqf, j) < most - kGtoNothing))
+                                gto_terms<double>(gt, pp, qq, pq, j, j + 1, g);
+                        auto fold = [](double& x) {
+                            x += xor_lane(x, kT);
+                            x += xor_lane(x, 2 * kT);
+                        };
+                        __syncwarp();
+                        fold(g.s0.re);
+                        fold(g.s0.im);
+                        fold(g.s1.re);
+                        fold(g.s1.im);
+                        if (gt.l == 1) {
+                            fold(g.s2.re);
+                            fold(g.s2.im);
+                            fold(g.s3.re);
+                            fold(g.s3.im);
+                        }
+                        if (valid && l == 0)
+                            contribution_closed<double>(v, gt, a.gamma, C, amp, Cx<double>{cs, -sn}, Cx<double>{cs_o, sn_o},
+                                                        g, cl, cv);
+                    }
                     __syncwarp();
-                    fold(g.s0.re);
-                    fold(g.s0.im);
-                    fold(g.s1.re);
-                    fold(g.s1.im);
-                    if (gt.l == 1) {
-                        fold(g.s2.re);
-                        fold(g.s2.im);
-                        fold(g.s3.re);
-                        fold(g.s3.im);
-                    }
-                    if (valid && l == 0)
-                        contribution_closed<double>(v, gt, a.gamma, C, amp, Cx<double>{cs, -sn}, Cx<double>{cs_o, sn_o},
-                                                    g, cl, cv);
-                }
-                __syncwarp();
 #pragma unroll
-                for (int o = 4; o > 0; o >>= 1) {   // over the trajectories (lanes 0..7 hold them)
-                    cl += xor_lane(cl, o);
-                    cv += xor_lane(cv, o);
+                    for (int o = 4; o > 0; o >>= 1) {   // over the trajectories (lanes 0..7 hold them)
+                        cl += xor_lane(cl, o);
+                        cv += xor_lane(cv, o);
+                    }
+                    if ((threadIdx.x & 31) == 0 && k_bin < f.n_bins && (cl != 0.0 || cv != 0.0)) {
+                        atomicAdd(&a.d_len[k_bin], cl);
+                        atomicAdd(&a.d_vel[k_bin], cv);
+                    }
                 }
-                if ((threadIdx.x & 31) == 0 && k_bin < f.n_bins && (cl != 0.0 || cv != 0.0)) {
-                    atomicAdd(&a.d_len[k_bin], cl);
-                    atomicAdd(&a.d_vel[k_bin], cv);
-                }
+                ++k_bin;
             }
-            ++k_bin;
+            alive_out[t] = alive ? 1 : 0;
+            rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
+            if constexpr (FB) {
+                // the step n -> n + 1: det Z of the advanced columns
+                const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, l & 1);
+                if (alive && n >= c.n0 && n < c.n_last) follow_branch<double>(Dp, D, sgn, flags);
+            } else {
+                if (c.have && n >= c.n0 && n < c.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, f.k64.h6);
+            }
+            if (alive && n >= c.n0 && n < c.n_last) {
+                ++all_steps;
+                if (n >= c.k_cnt) ++steps;
+            }
         }
-        alive_out[t] = alive ? 1 : 0;
-        rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
-        if constexpr (FB) {
-            // the step n -> n + 1: det Z of the advanced columns
-            const Cx2<double> D = det8(X0, X1, Y0, Y1, w, gz, qz, t, l & 1);
-            if (alive && n >= c.n0 && n < c.n_last) follow_branch<double>(Dp, D, sgn, flags);
-        } else {
-            if (c.have && n >= c.n0 && n < c.n_last) S += TrajP<double, POT>::action_sum(k1, k2, k3, k4, f.k64.h6);
-        }
-        if (alive && n >= c.n0 && n < c.n_last) {
-            ++all_steps;
-            if (n >= c.k_cnt) ++steps;
-        }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     if (a.stats) {
         const bool one = l == 0;   // a trajectory is counted by its first lane
@@ -634,7 +642,7 @@ __device__ void quad_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     }
     c.n_first = m;
     if (warp == 0 && c.l == 0) sm.alive[c.t] = c.alive0 ? 1 : 0;
-    if (threadIdx.x == 0) sm.last = c.n_last;
+    if (threadIdx.x == 0) sm.last = -1;
     __syncthreads();
     const int role = (warp + (int)(g & 3)) & 3;
     if (role == 0) quad_dynamics<POT, FB>(f, tg, a, c, sm);

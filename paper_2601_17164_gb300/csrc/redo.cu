@@ -66,7 +66,7 @@ struct Shared {
     double s12[2][kS12][kW];
     double s23[2][kS23][kW];
     int alive[kW];   // written by the bins warp, read late and without order by the warps ahead
-    long long last;  // the group's last grid point (GroupEnd)
+    long long last;  // the group's last grid point when it ends early, else -1 (GroupEnd)
 };
 
 struct Common {
@@ -95,42 +95,44 @@ __device__ void run_dynamics(const FieldDev& f, const TargetDev& tg, const TrajA
     double e0 = e_at(2 * c.n_first), e1 = e_at(2 * c.n_first + 1), e2 = e_at(2 * c.n_first + 2);
     const volatile int* alive = sm.alive;
     Producer<2> out(kHand0);
-    GroupEnd end(sm.last);
-    for (int64_t n = c.n_first; n <= end.last; ++n) {
-        {
-            const int d = out.acquire();
-            const bool live = alive[lane];
-            end.decide(n, live);
-            double* o = &sm.s01[d][0][lane];
-            o[29 * kW] = T.q[0];
-            o[30 * kW] = T.q[2];
-            o[31 * kW] = T.p[0];
-            o[32 * kW] = T.p[2];
-            // the E values of the next step, loaded one step ahead
-            const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
-            const bool step = c.have && n >= c.n0 && n < c.n_last && live;
-            if (step) {
-                double qs[4][2], gs[4], hs[4], ps[4][2], Vs[4];
-                T.stages_qp(e0, e1, e2, hk, pc, qs, gs, hs, ps, Vs);
+    for (int64_t n = c.n_first; n <= c.n_last;) {
+        int left = GroupEnd::stretch(n, c.n_last);
+        GroupEnd::decide(sm.last, n + left - 1, alive[lane]);
+        for (; left > 0; --left, ++n) {
+            {
+                const int d = out.acquire();
+                double* o = &sm.s01[d][0][lane];
+                o[29 * kW] = T.q[0];
+                o[30 * kW] = T.q[2];
+                o[31 * kW] = T.p[0];
+                o[32 * kW] = T.p[2];
+                // the E values of the next step, loaded one step ahead
+                const double f0 = e_at(2 * n + 2), f1 = e_at(2 * n + 3), f2 = e_at(2 * n + 4);
+                const bool step = c.have && n >= c.n0 && n < c.n_last && alive[lane];
+                if (step) {
+                    double qs[4][2], gs[4], hs[4], ps[4][2], Vs[4];
+                    T.stages_qp(e0, e1, e2, hk, pc, qs, gs, hs, ps, Vs);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    o[(2 * k) * kW] = qs[k][0];
-                    o[(2 * k + 1) * kW] = qs[k][1];
-                    o[(8 + k) * kW] = gs[k];
-                    o[(12 + k) * kW] = hs[k];
-                    o[(22 + k) * kW] = Vs[k];
-                }
+                    for (int k = 0; k < 4; ++k) {
+                        o[(2 * k) * kW] = qs[k][0];
+                        o[(2 * k + 1) * kW] = qs[k][1];
+                        o[(8 + k) * kW] = gs[k];
+                        o[(12 + k) * kW] = hs[k];
+                        o[(22 + k) * kW] = Vs[k];
+                    }
 #pragma unroll
-                for (int k = 1; k < 4; ++k) {
-                    o[(14 + 2 * k) * kW] = ps[k][0];
-                    o[(15 + 2 * k) * kW] = ps[k][1];
+                    for (int k = 1; k < 4; ++k) {
+                        o[(14 + 2 * k) * kW] = ps[k][0];
+                        o[(15 + 2 * k) * kW] = ps[k][1];
+                    }
                 }
+                out.publish(d);
+                e0 = f0;
+                e1 = f1;
+                e2 = f2;
             }
-            out.publish(d);
-            e0 = f0;
-            e1 = f1;
-            e2 = f2;
         }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -142,43 +144,45 @@ __device__ void run_matrix(const FieldDev& f, const Common& c, Shared& sm, int l
     const StepK<double> hk = f.k64;
     Consumer<2> in_q(kHand0);
     Producer<2> out(kHand1);
-    GroupEnd end(sm.last);
-    for (int64_t n = c.n_first; n <= end.last; ++n) {
-        {
-            const int di = in_q.wait();
-            end.follow();
-            const int dq = out.acquire();
-            const double* in = &sm.s01[di][0][lane];
-            double* o = &sm.s12[dq][0][lane];
+    for (int64_t n = c.n_first; n <= c.n_last;) {
+        int left = GroupEnd::stretch(n, c.n_last);
+        for (; left > 0; --left, ++n) {
+            {
+                const int di = in_q.wait();
+                const int dq = out.acquire();
+                const double* in = &sm.s01[di][0][lane];
+                double* o = &sm.s12[dq][0][lane];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o[(19 + k) * kW] = in[(29 + k) * kW];
-            if (c.have && n >= c.n0 && n < c.n_last) {
-                double qs[4][2], gs[4], hs[4];
+                for (int k = 0; k < 4; ++k) o[(19 + k) * kW] = in[(29 + k) * kW];
+                if (c.have && n >= c.n0 && n < c.n_last) {
+                    double qs[4][2], gs[4], hs[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    qs[k][0] = in[(2 * k) * kW];
-                    qs[k][1] = in[(2 * k + 1) * kW];
-                    gs[k] = in[(8 + k) * kW];
-                    hs[k] = in[(12 + k) * kW];
+                    for (int k = 0; k < 4; ++k) {
+                        qs[k][0] = in[(2 * k) * kW];
+                        qs[k][1] = in[(2 * k + 1) * kW];
+                        gs[k] = in[(8 + k) * kW];
+                        hs[k] = in[(12 + k) * kW];
+                    }
+                    const StepMat<double> M = TrajP<double, POT>::step_matrix(qs, gs, hs, hk);
+#pragma unroll
+                    for (int k = 0; k < 15; ++k) o[k * kW] = M.m[k];   // (its out-of-plane part is left out)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) o[(15 + k) * kW] = gs[k];
+                    // the action increment's inputs
+#pragma unroll
+                    for (int k = 1; k < 4; ++k) {
+                        o[(22 + k) * kW] = qs[k][1];
+                        o[(24 + 2 * k) * kW] = in[(14 + 2 * k) * kW];
+                        o[(25 + 2 * k) * kW] = in[(15 + 2 * k) * kW];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) o[(32 + k) * kW] = in[(22 + k) * kW];
                 }
-                const StepMat<double> M = TrajP<double, POT>::step_matrix(qs, gs, hs, hk);
-#pragma unroll
-                for (int k = 0; k < 15; ++k) o[k * kW] = M.m[k];   // (its out-of-plane part is left out)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) o[(15 + k) * kW] = gs[k];
-                // the action increment's inputs
-#pragma unroll
-                for (int k = 1; k < 4; ++k) {
-                    o[(22 + k) * kW] = qs[k][1];
-                    o[(24 + 2 * k) * kW] = in[(14 + 2 * k) * kW];
-                    o[(25 + 2 * k) * kW] = in[(15 + 2 * k) * kW];
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) o[(32 + k) * kW] = in[(22 + k) * kW];
+                in_q.release(di);
+                out.publish(dq);
             }
-            in_q.release(di);
-            out.publish(dq);
         }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -195,56 +199,58 @@ __device__ void run_columns(const FieldDev& f, const Common& c, Shared& sm, int 
     const volatile int* alive = sm.alive;
     Consumer<2> in_q(kHand1);
     Producer<2> out(kHand2);
-    GroupEnd end(sm.last);
-    for (int64_t n = c.n_first; n <= end.last; ++n) {
-        {
-            const int di = in_q.wait();
-            end.follow();
-            const int dq = out.acquire();
-            const double* in = &sm.s12[di][0][lane];
-            double* o = &sm.s23[dq][0][lane];
-            const double s_n = S.value();   // the action at grid point n
-            if (c.have && n >= c.n0 && n < c.n_last && alive[lane]) {
-                StepMat<double> M;
+    for (int64_t n = c.n_first; n <= c.n_last;) {
+        int left = GroupEnd::stretch(n, c.n_last);
+        for (; left > 0; --left, ++n) {
+            {
+                const int di = in_q.wait();
+                const int dq = out.acquire();
+                const double* in = &sm.s12[di][0][lane];
+                double* o = &sm.s23[dq][0][lane];
+                const double s_n = S.value();   // the action at grid point n
+                if (c.have && n >= c.n0 && n < c.n_last && alive[lane]) {
+                    StepMat<double> M;
 #pragma unroll
-                for (int k = 0; k < 15; ++k) M.m[k] = in[k * kW];
+                    for (int k = 0; k < 15; ++k) M.m[k] = in[k * kW];
 #pragma unroll
-                for (int k = 15; k < 19; ++k) M.m[k] = 0.0;   // the bins warp advances the out-of-plane block
-                T.apply_step_matrix(M);
-            }
-            if (c.have && n >= c.n0 && n < c.n_last) {
-                double qs[4][2], ps[4][2], Vs[4];
-                qs[0][1] = in[20 * kW];   // the state at n: q_z, p_x', p_z
-                ps[0][0] = in[21 * kW];
-                ps[0][1] = in[22 * kW];
+                    for (int k = 15; k < 19; ++k) M.m[k] = 0.0;   // the bins warp advances the out-of-plane block
+                    T.apply_step_matrix(M);
+                }
+                if (c.have && n >= c.n0 && n < c.n_last) {
+                    double qs[4][2], ps[4][2], Vs[4];
+                    qs[0][1] = in[20 * kW];   // the state at n: q_z, p_x', p_z
+                    ps[0][0] = in[21 * kW];
+                    ps[0][1] = in[22 * kW];
 #pragma unroll
-                for (int k = 1; k < 4; ++k) {
-                    qs[k][1] = in[(22 + k) * kW];
-                    ps[k][0] = in[(24 + 2 * k) * kW];
-                    ps[k][1] = in[(25 + 2 * k) * kW];
+                    for (int k = 1; k < 4; ++k) {
+                        qs[k][1] = in[(22 + k) * kW];
+                        ps[k][0] = in[(24 + 2 * k) * kW];
+                        ps[k][1] = in[(25 + 2 * k) * kW];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        qs[k][0] = 0.0;   // not read by the action terms
+                        Vs[k] = in[(32 + k) * kW];
+                    }
+                    auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(f.E64 + j) : 0.0; };
+                    S.add(TrajP<double, POT>::action_increment(ps, qs, Vs, e_at(2 * n), e_at(2 * n + 1), e_at(2 * n + 2),
+                                                               h6));
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    qs[k][0] = 0.0;   // not read by the action terms
-                    Vs[k] = in[(32 + k) * kW];
+                    o[(4 * k) * kW] = T.X[k][0];
+                    o[(4 * k + 1) * kW] = T.X[k][1];
+                    o[(4 * k + 2) * kW] = T.Y[k][0];
+                    o[(4 * k + 3) * kW] = T.Y[k][1];
                 }
-                auto e_at = [&](int64_t j) { return j < f.table_len ? __ldg(f.E64 + j) : 0.0; };
-                S.add(TrajP<double, POT>::action_increment(ps, qs, Vs, e_at(2 * n), e_at(2 * n + 1), e_at(2 * n + 2),
-                                                           h6));
-            }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                o[(4 * k) * kW] = T.X[k][0];
-                o[(4 * k + 1) * kW] = T.X[k][1];
-                o[(4 * k + 2) * kW] = T.Y[k][0];
-                o[(4 * k + 3) * kW] = T.Y[k][1];
+                for (int k = 0; k < 8; ++k) o[(16 + k) * kW] = in[(15 + k) * kW];   // g of the stages, state
+                o[24 * kW] = s_n;
+                in_q.release(di);
+                out.publish(dq);
             }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) o[(16 + k) * kW] = in[(15 + k) * kW];   // g of the stages, state
-            o[24 * kW] = s_n;
-            in_q.release(di);
-            out.publish(dq);
         }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     out.drain();
 }
@@ -326,102 +332,104 @@ __device__ void run_bins(const FieldDev& f, const TargetDev& tg, const GtoTerms&
     int64_t k_next = (c.n_first + c.n_out - 1) / c.n_out;   // bin index of the next output point
     volatile int* alive_out = sm.alive;
     Consumer<2> in_q(kHand2);
-    GroupEnd end(sm.last);
-    for (int64_t n = c.n_first; n <= end.last; ++n) {
-        {
-            const int di = in_q.wait();
-            end.follow();
-            const double* in = &sm.s23[di][0][lane];
-            const double q0 = in[20 * kW], q2 = in[21 * kW], p0 = in[22 * kW], p2 = in[23 * kW], S = in[24 * kW];
-            const bool on_bin = rem == 0;
-            // partial waves (Sec. III.A-B): class at each entry into r < R, labels at
-            // every grid point from birth on while the trajectory is integrated
-            if (pw && alive && n >= c.n0) {
-                const double qx = q0, qy = 0.0, qz = q2;
-                const bool inside = qx * qx + qy * qy + qz * qz < pw_r2;
-                if (inside && !pw_in) {
-                    const double px = p0, py = 0.0, pz = p2;
-                    const double lx = qy * pz - qz * py, ly = qz * px - qx * pz, lz = qx * py - qy * px;
-                    const double L2 = lx * lx + ly * ly + lz * lz;
-                    pw_cls = L2 < 0.25 ? 0 : (L2 < 2.25 ? 1 : (L2 < 6.25 ? 2 : 3));
+    for (int64_t n = c.n_first; n <= c.n_last;) {
+        int left = GroupEnd::stretch(n, c.n_last);
+        for (; left > 0; --left, ++n) {
+            {
+                const int di = in_q.wait();
+                const double* in = &sm.s23[di][0][lane];
+                const double q0 = in[20 * kW], q2 = in[21 * kW], p0 = in[22 * kW], p2 = in[23 * kW], S = in[24 * kW];
+                const bool on_bin = rem == 0;
+                // partial waves (Sec. III.A-B): class at each entry into r < R, labels at
+                // every grid point from birth on while the trajectory is integrated
+                if (pw && alive && n >= c.n0) {
+                    const double qx = q0, qy = 0.0, qz = q2;
+                    const bool inside = qx * qx + qy * qy + qz * qz < pw_r2;
+                    if (inside && !pw_in) {
+                        const double px = p0, py = 0.0, pz = p2;
+                        const double lx = qy * pz - qz * py, ly = qz * px - qx * pz, lz = qx * py - qy * px;
+                        const double L2 = lx * lx + ly * ly + lz * lz;
+                        pw_cls = L2 < 0.25 ? 0 : (L2 < 2.25 ? 1 : (L2 < 6.25 ? 2 : 3));
+                    }
+                    pw_in = inside;
                 }
-                pw_in = inside;
-            }
-            const bool pw_ok = !pw || (pw_cls >= 0 && ((a.pw_mask >> pw_cls) & 1));
-            if (on_bin) {
-                if (pending) finish();
-                valid = false;
-                if (alive && n >= c.n0) {
-                    const double fs = q0 + q2 + p0 + p2;
-                    const bool ok = isfinite(fs) && isfinite(S);
-                    const cd D = 0.125 * cd{Dp.re, Dp.im};
-                    const double m2 = D.re * D.re + D.im * D.im;
-                    if (!ok || !(m2 <= a.d_t * a.d_t)) {
-                        alive = false;
-                        flags |= 1u;
-                        if (!ok || !isfinite(m2)) flags |= 2u;
-                    } else if (n >= c.k_cnt && pw_ok) {
-                        cd Cz = root_det(D, m2);
-                        if (sgn < 0.0) Cz = -Cz;
-                        C = Cx<double>{Cz.re, Cz.im};
-                        valid = true;
-                        bq0 = q0;
-                        bq2 = q2;
-                        bp0 = p0;
-                        bp2 = p2;
-                        bS = S;
-                        if (fbins)
-                            recomb_invariants<float>(FloatState(bq0, 0.0, bq2, bp0, 0.0, bp2, bS), p2f, q2f, pqf);
-                        else {
-                            recomb_invariants<double>(PView(bq0, bq2, bp0, bp2, bS), p2s, q2s, pqs);
-                            p2f = (float)p2s;
-                            q2f = (float)q2s;
-                            most = -INFINITY;
-                            for (int j = 0; j < gt.n; ++j) most = fmaxf(most, gto_size(gt, p2f, q2f, j));
+                const bool pw_ok = !pw || (pw_cls >= 0 && ((a.pw_mask >> pw_cls) & 1));
+                if (on_bin) {
+                    if (pending) finish();
+                    valid = false;
+                    if (alive && n >= c.n0) {
+                        const double fs = q0 + q2 + p0 + p2;
+                        const bool ok = isfinite(fs) && isfinite(S);
+                        const cd D = 0.125 * cd{Dp.re, Dp.im};
+                        const double m2 = D.re * D.re + D.im * D.im;
+                        if (!ok || !(m2 <= a.d_t * a.d_t)) {
+                            alive = false;
+                            flags |= 1u;
+                            if (!ok || !isfinite(m2)) flags |= 2u;
+                        } else if (n >= c.k_cnt && pw_ok) {
+                            cd Cz = root_det(D, m2);
+                            if (sgn < 0.0) Cz = -Cz;
+                            C = Cx<double>{Cz.re, Cz.im};
+                            valid = true;
+                            bq0 = q0;
+                            bq2 = q2;
+                            bp0 = p0;
+                            bp2 = p2;
+                            bS = S;
+                            if (fbins)
+                                recomb_invariants<float>(FloatState(bq0, 0.0, bq2, bp0, 0.0, bp2, bS), p2f, q2f, pqf);
+                            else {
+                                recomb_invariants<double>(PView(bq0, bq2, bp0, bp2, bS), p2s, q2s, pqs);
+                                p2f = (float)p2s;
+                                q2f = (float)q2s;
+                                most = -INFINITY;
+                                for (int j = 0; j < gt.n; ++j) most = fmaxf(most, gto_size(gt, p2f, q2f, j));
+                            }
                         }
                     }
+                    k_bin = k_next++;
+                    pending = true;
+                    j_next = 0;
+                    acc = GtoSums<double>{};
+                    accf = GtoSums<float>{};
                 }
-                k_bin = k_next++;
-                pending = true;
-                j_next = 0;
-                acc = GtoSums<double>{};
-                accf = GtoSums<float>{};
-            }
-            // the step n -> n + 1: det Z of the advanced columns and its branch
-            if (alive && n >= c.n0 && n < c.n_last) {
+                // the step n -> n + 1: det Z of the advanced columns and its branch
+                if (alive && n >= c.n0 && n < c.n_last) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    T.X[k][0] = in[(4 * k) * kW];
-                    T.X[k][1] = in[(4 * k + 1) * kW];
-                    T.Y[k][0] = in[(4 * k + 2) * kW];
-                    T.Y[k][1] = in[(4 * k + 3) * kW];
+                    for (int k = 0; k < 4; ++k) {
+                        T.X[k][0] = in[(4 * k) * kW];
+                        T.X[k][1] = in[(4 * k + 1) * kW];
+                        T.Y[k][0] = in[(4 * k + 2) * kW];
+                        T.Y[k][1] = in[(4 * k + 3) * kW];
+                    }
+                    // the out-of-plane block, H_s = g_s (TrajP::step_matrix and apply_step_matrix)
+                    const double g0 = in[16 * kW], g1 = in[17 * kW], g2 = in[18 * kW], g3 = in[19 * kW];
+                    const double g23 = g1 + g2;
+                    const double oa = fma(hk.c4, g2 * g0, -hk.c2 * (g23 + g0)), ob = fma(-hk.c3, g23, hk.h);
+                    const double oc = fma(hk.c3, fma(g2, g0, g3 * g1), -hk.h6 * (fma(2.0, g23, g0) + g3));
+                    const double od = fma(hk.c4, g3 * g1, -hk.c2 * (g23 + g3));
+                    const double ya = T.aq, pa = T.ap, yb = T.bq, pb = T.bp;
+                    T.aq = fma(oa, ya, fma(ob, pa, ya));
+                    T.ap = fma(oc, ya, fma(od, pa, pa));
+                    T.bq = fma(oa, yb, fma(ob, pb, yb));
+                    T.bp = fma(oc, yb, fma(od, pb, pb));
+                    const Cx2<double> D = T.detc(1.0, -2.0 * rg, 2.0 * a.qg64);
+                    follow_branch<double>(Dp, D, sgn, flags);
+                    ++all_steps;
+                    if (n >= c.k_cnt) ++steps;
                 }
-                // the out-of-plane block, H_s = g_s (TrajP::step_matrix and apply_step_matrix)
-                const double g0 = in[16 * kW], g1 = in[17 * kW], g2 = in[18 * kW], g3 = in[19 * kW];
-                const double g23 = g1 + g2;
-                const double oa = fma(hk.c4, g2 * g0, -hk.c2 * (g23 + g0)), ob = fma(-hk.c3, g23, hk.h);
-                const double oc = fma(hk.c3, fma(g2, g0, g3 * g1), -hk.h6 * (fma(2.0, g23, g0) + g3));
-                const double od = fma(hk.c4, g3 * g1, -hk.c2 * (g23 + g3));
-                const double ya = T.aq, pa = T.ap, yb = T.bq, pb = T.bp;
-                T.aq = fma(oa, ya, fma(ob, pa, ya));
-                T.ap = fma(oc, ya, fma(od, pa, pa));
-                T.bq = fma(oa, yb, fma(ob, pb, yb));
-                T.bp = fma(oc, yb, fma(od, pb, pb));
-                const Cx2<double> D = T.detc(1.0, -2.0 * rg, 2.0 * a.qg64);
-                follow_branch<double>(Dp, D, sgn, flags);
-                ++all_steps;
-                if (n >= c.k_cnt) ++steps;
+                in_q.release(di);
+                alive_out[lane] = alive ? 1 : 0;
+                rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
             }
-            in_q.release(di);
-            alive_out[lane] = alive ? 1 : 0;
-            rem = (rem + 1 == c.n_out) ? 0 : rem + 1;
+            if (pending) {
+                const int j_end = j_next + tps < gt.n ? j_next + tps : gt.n;
+                if (valid) terms(j_next, j_end);
+                j_next = j_end;
+                if (j_next >= gt.n) finish();
+            }
         }
-        if (pending) {
-            const int j_end = j_next + tps < gt.n ? j_next + tps : gt.n;
-            if (valid) terms(j_next, j_end);
-            j_next = j_end;
-            if (j_next >= gt.n) finish();
-        }
+        if (GroupEnd::here(sm.last, n - 1)) break;
     }
     if (pending) finish();
     if (a.stats) {
@@ -479,7 +487,7 @@ __device__ void redo_group(const FieldDev& f, const TargetDev& tg, const GtoTerm
     }
     c.n_first = m;
     if (warp == 0) sm.alive[lane] = c.alive0 ? 1 : 0;
-    if (threadIdx.x == 0) sm.last = c.n_last;
+    if (threadIdx.x == 0) sm.last = -1;
     __syncthreads();
     const int role = (warp + (int)(g & 3)) & 3;
     if (role == 0) run_dynamics<POT>(f, tg, a, c, sm, lane);

@@ -1,6 +1,7 @@
 // Pieces shared by the warp-specialised FP64 kernels (redo.cu, quad.cu): the hand-off
 // rings between the warps of a block, the view of a planar state that the
-// recombination terms take, the root of det Z, and where a block's groups come from.
+// recombination terms take, the root of det Z, where a block's groups come from and
+// where a group ends.
 #pragma once
 
 #include "traj_block.cuh"
@@ -78,22 +79,23 @@ struct Consumer {
     }
 };
 
-// The last grid point of a group, in shared memory: that of the call, until the bins warp
-// has removed every trajectory.  The dynamics warp, the first of the chain, learns of it
-// from the labels and makes the grid point that it is about to publish the last one; the
-// hand-offs order that write before the item, so each warp behind it reads it by the time
-// that it has waited for that item, and all four end on the same one.
+// A group runs in stretches of 8 grid points and ends early, at the end of a stretch, when
+// the bins warp has removed every trajectory.  The dynamics warp, the first of the chain,
+// learns of it from the labels: at the start of a stretch, before it publishes an item of
+// it, it marks that stretch as the last one.  The hand-offs order the mark before the items,
+// so each warp behind finds it when it is done with the stretch, and all four end on the
+// same one.  (Looking at every grid point costs a short list 2 %, nothing this way.)
 struct GroupEnd {
-    volatile long long* at;
-    int64_t last;
-    __device__ explicit GroupEnd(long long& shared) : at(&shared), last(shared) {}
-    __device__ void decide(int64_t n, bool alive) {   // by the dynamics warp, converged
-        if (!__any_sync(0xffffffffu, alive) && n < last) {
-            last = n;
-            if ((threadIdx.x & 31) == 0) *at = n;
-        }
+    static constexpr int kStretch = 8;
+    // grid points of the stretch that starts at n
+    static __device__ int stretch(int64_t n, int64_t n_last) {
+        return n_last - n + 1 < kStretch ? (int)(n_last - n + 1) : kStretch;
     }
-    __device__ void follow() { last = *at; }           // by the others, after the wait for an item
+    // by the dynamics warp, converged
+    static __device__ void decide(long long& mark, int64_t hi, bool alive) {
+        if (!__any_sync(0xffffffffu, alive) && (threadIdx.x & 31) == 0) *(volatile long long*)&mark = hi;
+    }
+    static __device__ bool here(const long long& mark, int64_t hi) { return *(const volatile long long*)&mark == hi; }
 };
 
 __device__ __forceinline__ unsigned sm_id() {
