@@ -81,27 +81,37 @@ def flops_per_traj_step(pot: int, planar: bool = True, compensated: bool = True)
     return float(qps + comp + cols + branch)
 
 
+def short_list(pot: int, sms: int) -> int:
+    """Longest escalation list of the four-lane FP64 kernel: 2 groups of 8 per SM, 5 for Tong-Lin."""
+    return 8 * sms * (5 if pot == W.POT_TONGLIN else 2)
+
+
 def launches_per_step(n: int, n_steps: int, chunk: int, prec: int, floor: bool, overlap: int = 0,
-                      block: int = 128, side: int = 8, esc_precision: int = 0) -> int:
+                      block: int = 128, side: int = 8, esc_precision: int = 0, short: int = None) -> int:
     """Our kernels per step: births, the trajectory pass(es), spectra (x2).  The mixed
     path with escalation (as sfhk_dipole runs it) adds the amplitude maximum and, per
     birth chunk (overlap 0) or time segment (overlap 1) of the float pass, or once
     (overlap 2, sequential), the float launch, two compaction kernels and the
-    high-precision redo (esc_precision 0, planar form: its one-warp group plan and the
-    launches for short and for long lists, of which one returns at once).  One too many
-    per part where esc_precision is 1 or 2, and where a part has no more births than a
-    short list holds (only the launch for short lists follows)."""
+    high-precision redo: one launch where esc_precision is 1 or 2; for esc_precision 0
+    (planar form) its one-warp group plan, the launch for short lists and, where a part has
+    more births than such a list (`short`, short_list), the one for long lists, of which
+    one returns at once.  Without `short`, the most that a step of these parts can launch
+    (one more per part than esc_precision 1 and 2 need)."""
     if prec != 1:
         return 1 + 1 + 2
     if overlap == 2:
-        parts = 1
+        parts = [n]
     elif overlap == 0:
         per = -(-n // side)
         csz = max(-(-per // block) * block, 64 * block)
-        parts = -(-n // csz)
+        parts = [min(csz, n - c) for c in range(0, n, csz)]
     else:
-        parts = min(side, (n_steps + chunk) // chunk)
-    return 1 + (1 if floor else 0) + parts * (6 if esc_precision == 0 else 5) + 2
+        parts = [n] * min(side, (n_steps + chunk) // chunk)
+    if short is None:
+        redo = len(parts) * (6 if esc_precision == 0 else 5)
+    else:
+        redo = sum(4 if esc_precision else (6 if p > short else 5) for p in parts)
+    return 1 + (1 if floor else 0) + redo + 2
 
 
 class Clocks:
@@ -463,6 +473,7 @@ def gpu_arm(args):
 
     if rank == 0:
         kms = statistics.mean(kern_ms)
+        short = short_list(w.target.pot, torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count)
         peak32 = 2 * FP32_LANES_PER_SM * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
         peak64 = 2 * FP64_LANES_PER_SM * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
         f64_fps = flops_per_traj_step(w.target.pot, planar=True, compensated=False)
@@ -509,7 +520,9 @@ def gpu_arm(args):
         else:
             ach = f64_fps * steps_per_launch / (kms * 1e-3) / 1e12
             roofline = {"bound": "alu", "achieved": ach, "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64,
-                        "traffic": None, "kernel": "traj_kernel<double,SOFTCORE,planar>", "kernel_ms": kms,
+                        "traffic": None, "kernel_ms": kms,
+                        "kernel": ("traj_kernel<double,SOFTCORE,planar>" if args.block or args.chunk else
+                                   "quad_kernel<SOFTCORE, FP64 bins>" if w.n <= short else "redo_kernel<SOFTCORE>"),
                         "flops_per_traj_step": f64_fps,
                         "peak_basis": "152 SMs x 2 FP64 lanes x 2 flops x 2070 MHz (of nominal)"}
         roofline = dict(roofline, dipole_call_ms=kms)
@@ -538,9 +551,10 @@ def gpu_arm(args):
             "measured_peaks": peaks,
             "fp64_path": fp64,
             "e2e": e2e,
-            "gpu_launches": launches_per_step(w.n, info["n_steps"], args.chunk or 1000, prec,
+            "gpu_launches": launches_per_step(w.n, info["n_steps"], args.chunk or 1000,
+                                              prec if pp.esc_ratio > 0.0 else 0,
                                               pp.esc_floor > 0.0, pp.esc_overlap,
-                                              esc_precision=pp.esc_precision) * args.steps,
+                                              esc_precision=pp.esc_precision, short=short) * args.steps,
             "clocks": clk,
             "wall_s": wall,
         }
