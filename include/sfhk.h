@@ -419,9 +419,12 @@ sfhk_status sfhk_get_phase_times(sfhk_phase_times* out);
  * windows of 25, 50, 100, 200 and 400 output bins (chunk_steps = bins * n_out,
  * which also sets the shared-memory bin tile), escalation off, one warm-up and
  * one timed run each; keeps the fastest for (device, precision, planar form,
- * potential).  Later calls with block = chunk_steps = 0 use it (FP64 planar dipoles
- * into atomic bins run on kernels without such a shape).  Writes the
- * choice to best_block / best_chunk / best_ms (host pointers, may be NULL).
+ * potential).  Later calls with block = chunk_steps = 0 use it where they run on
+ * the one-thread-per-trajectory kernel: not FP64 endpoints and FP64 planar
+ * dipoles into atomic bins (see block above), whose kernels have no such shape.
+ * For the latter that default call is timed too, and where it is the faster one
+ * the choice is 0, 0 and its time.  Writes the choice to best_block / best_chunk /
+ * best_ms (host pointers, may be NULL).
  * Synchronous; allocates 2 n_bins doubles for the duration of the call.
  * ---------------------------------------------------------------------- */
 sfhk_status sfhk_autotune(const sfhk_field* field, const sfhk_target* target, const sfhk_births* births,

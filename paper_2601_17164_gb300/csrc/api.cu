@@ -941,6 +941,17 @@ sfhk_status sfhk_autotune(const sfhk_field* field, const sfhk_target* target, co
     const int chunk_bins[5] = {25, 50, 100, 200, 400};
     float best = 1e30f;
     int bb = 128, bc = 100;
+    auto run_once = [&](const sfhk_prop_params& pp) {
+        float ms = 0.f;
+        for (int rep = 0; rep < 2 && !st; ++rep) {   // warm-up, then timed
+            cudaEventRecord(e0, s);
+            st = sfhk_dipole(field, target, births, n_sample, &pp, bins, bins + nb, nullptr, stream);
+            cudaEventRecord(e1, s);
+            if (!st) st = check_cuda(cudaEventSynchronize(e1), "autotune sync");
+            if (!st) cudaEventElapsedTime(&ms, e0, e1);
+        }
+        return ms;
+    };
     for (int ib = 0; ib < 2 && !st; ++ib)
         for (int ic = 0; ic < 5 && !st; ++ic) {
             sfhk_prop_params pp = *params;
@@ -949,27 +960,36 @@ sfhk_status sfhk_autotune(const sfhk_field* field, const sfhk_target* target, co
             pp.esc_ratio = 0.0;
             pp.deterministic = 0;
             if (pp.chunk_steps < 64 || pp.chunk_steps > 8192) continue;
-            float ms = 0.f;
-            for (int rep = 0; rep < 2 && !st; ++rep) {   // warm-up, then timed
-                cudaEventRecord(e0, s);
-                st = sfhk_dipole(field, target, births, n_sample, &pp, bins, bins + nb, nullptr, stream);
-                cudaEventRecord(e1, s);
-                if (!st) st = check_cuda(cudaEventSynchronize(e1), "autotune sync");
-                if (!st) cudaEventElapsedTime(&ms, e0, e1);
-            }
+            const float ms = run_once(pp);
             if (!st && ms < best) {
                 best = ms;
                 bb = blocks[ib];
                 bc = chunk_bins[ic];
             }
         }
+    // An FP64 planar dipole into atomic bins takes no shape by default (run_traj): where that
+    // call is the faster one, it is the choice (block = chunk_steps = 0); the best shape is
+    // still kept for the calls that use one.
+    const int planar = (births->q0x == nullptr && births->q0y == nullptr && params->geometry == 0) ? 1 : 0;
+    bool shape = true;
+    if (!st && params->precision == 0 && planar && !params->deterministic && params->d_t <= kWarpsDt &&
+        n_sample <= fp64_limit(target->t.pot, redo_lists())) {
+        sfhk_prop_params pp = *params;
+        pp.block = pp.chunk_steps = 0;
+        pp.esc_ratio = 0.0;
+        pp.deterministic = 0;
+        const float ms = run_once(pp);
+        if (!st && ms < best) {
+            best = ms;
+            shape = false;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFree(bins);
     if (st) return st;
     int dev;
     cudaGetDevice(&dev);
-    const int planar = (births->q0x == nullptr && births->q0y == nullptr && params->geometry == 0) ? 1 : 0;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         bool found = false;
@@ -981,8 +1001,8 @@ sfhk_status sfhk_autotune(const sfhk_field* field, const sfhk_target* target, co
             }
         if (!found) g_tuned.push_back(Tuned{dev, params->precision, planar, target->t.pot, bb, bc});
     }
-    if (best_block) *best_block = bb;
-    if (best_chunk) *best_chunk = bc * n_out;
+    if (best_block) *best_block = shape ? bb : 0;
+    if (best_chunk) *best_chunk = shape ? bc * n_out : 0;
     if (best_ms) *best_ms = best;
     return SFHK_OK;
 }
