@@ -2,7 +2,8 @@
 // App. B.1 tunnelling matrix elements; App. B.2 modified SPA; Sec. III.C ADK
 // births renormalised to the SFA rate at the pulse's two sub-peaks).
 //
-// One thread per birth, FP64.  The birth draws (grid or Philox) are integer
+// FP64, a thread for each birth's draw and bracket and for its amplitude, the roots in
+// between from a queue.  The birth draws (grid or Philox) are integer
 // exact; the saddle point is the smallest t_t > 0 with
 // Im A(t0 + i t_t) = s kappa, s = -sign E(t0), found by a scan for the first grid
 // cell with a sign change, then a Newton iteration kept inside the bracket

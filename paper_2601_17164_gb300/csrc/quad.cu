@@ -20,13 +20,13 @@
 // det Z (lane j forms column j of Z, even lanes the real and odd lanes the imaginary part)
 // goes to the bins warp when the recombination terms are formed in float, to the columns
 // warp when FP64 terms load the bins warp.
-// FP64 instructions per step: dynamics 84 -> 29 (soft-core), 380 -> 111 (Tong-Lin), the
-// four warps 29, 28, 33, 29 (float bins, soft-core): a block alone on its SM steps in
-// 2,900 cycles instead of the 7,600 of 32 trajectories a block (Tong-Lin: 8,500 instead
-// of 24,200), with 1.5 times the FP64 work per trajectory, so the host and the plan
-// choose by list length (quad_limit).  Measured: mixed H 8 cycles, 4096 births (110
-// redone) 334 -> 170 ms; mixed Ar 6 cycles, 5e4 births 1730 -> 660 ms; FP64 H 2 cycles,
-// 1024 births 140.6 -> 21.3 ms.
+// FP64 instructions of the longest chain, the dynamics: 84 -> 29 a step (soft-core), 380 ->
+// 111 (Tong-Lin); of all four warps 114 and 211 (ncu, FP64 bins left out).  A block alone on
+// its SM steps in 2,900 cycles (float bins; FP64 3,800) where 32 trajectories a block take
+// 6,300 (Tong-Lin: 8,000 to 8,500 and 24,700), with 1.5 times the FP64 work per trajectory,
+// so the host and the plan choose by list length (quad_limit).  Measured: mixed H 8 cycles,
+// 4096 births (110 redone) 333 -> 169 ms; mixed Ar 6 cycles, 5e4 births 1730 -> 650 ms; FP64
+// H 2 cycles, 1024 births 143 -> 22 ms.
 //
 // Every value is formed by the same operations in the same order as in TrajP
 // (traj_block.cuh): trajectories, columns, determinants, branches and removals are

@@ -18,19 +18,21 @@
 //             partial-wave labels, removal and the prefactor at the bins, and
 //             the GTO recombination sums, spread over the steps between bins,
 //             with the warp reduction and the atomic bin update.
-// The warps form a pipeline one grid point apart, handing data on through
-// double-buffered shared-memory slots with one CTA barrier per grid point.
+// The warps form a pipeline, each handing data on to the next through two slots in
+// shared memory on named barriers of the two warps (redo_warps.cuh), so that a warp can
+// run up to two grid points ahead of the next one.
 // The roles rotate with the block index so that the heavier roles of the
 // blocks resident on one SM spread over its four sub-partitions.  Removal is
 // decided by the bins warp; the warps ahead of it learn of it a few grid
 // points late and only skip work that no longer counts.
 //
 // Lists long enough to fill the chip at 32 trajectories a block come here (quad_limit);
-// then the FP64 instructions of all roles decide, 19 cycles of the SM each: 84, 79, 84 and
-// 44 per step (soft-core), of which the branch's comparisons on the bits of doubles and
-// 8 det Z of 2 Z (no halves) saved 15.  Measured, mixed H 8 cycles, 1e6 births (12,200
-// redone): 496 -> 473 ms; FP64 H 1600 nm 3 cycles, 20011 births: 471 ms with one thread per
-// trajectory, 242 ms here (271 ms with every GTO term of every bin).
+// then the FP64 instructions of all roles decide, 19 cycles of the SM each: 301 per step of
+// a group, bins left out (soft-core; Tong-Lin 604; ncu), 15 fewer since the branch compares
+// the bits of doubles and follows 8 det Z of 2 Z (no halves).  Measured, mixed H 8 cycles,
+// 1e6 births (12,200 redone): 496 -> 472 ms; FP64 H 1600 nm 3 cycles, 20011 births: 471 to
+// 483 ms with one thread per trajectory, 237 to 287 ms here by the sample (271 instead of
+// 242 ms with every GTO term of every bin).
 //
 // Each part runs the same device functions as the one-thread-per-trajectory
 // kernel (TrajP::stages_qp / action_term / action_sum, TrajP::step_matrix,
@@ -613,8 +615,6 @@ cudaError_t launch_wide(const FieldDev& f, const TargetDev& t, const TrajArgs& a
 
 }  // namespace
 
-int64_t redo_blocks(int64_t n) { return (n + kW - 1) / kW; }
-
 int redo_lists() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 1;
@@ -622,11 +622,15 @@ int redo_lists() {
     return std::max(1, std::min(sms, kRedoLists));
 }
 
-// Longest list for the four-lane kernel, from FP64 instructions per step (64 cycles each on
-// the longest role, 19 per SM for all roles): with m groups of 8 per SM it steps in about
-// max(2,900, m x 122 x 19) cycles (soft-core), the 32-wide kernel with one group per SM in
-// 6,400: two groups of 8 per SM win (4,600), three do not (7,000).  Tong-Lin: max(8,500, m
-// x 216 x 19) against 24,000: five do.
+// Longest list for the four-lane kernel.  Set by FP64 instructions per step of a group, 64
+// cycles each on the longest role and 19 of the SM for all roles: m groups of 8 per SM take
+// at least m x 114 x 19 cycles (soft-core; Tong-Lin m x 211 x 19), one group of 32 takes 6,300
+// (24,700).  Measured on both sides, 800 nm 1 cycle, 152 SMs, bins every fifth step:
+//   lists, float bins     soft-core  9.2 ms at 2175 entries, 32-wide 17.7 ms at 2507;
+//                         Tong-Lin  29.7 ms at 5369, 64.2 ms at 6191;
+//   FP64 calls and bins   soft-core 10.6 ms at 2432, 26.5 ms at 2433;
+//                         harmonic  10.9 and 30.2 ms; Tong-Lin 29.3 ms at 6080, 66.0 ms at 6081.
+// The lines lie on the safe side of where the two meet.
 int64_t quad_limit(int pot, int lists) { return (int64_t)kQuadWidth * lists * (pot == POT_TONGLIN ? 5 : 2); }
 
 // Longest FP64 dipole call for the warp-specialised kernels.  The harmonic force leaves the

@@ -109,7 +109,7 @@ __device__ __forceinline__ unsigned sm_id() {
 // one atomic counter per list.  A block that finds its own list empty waits 20 us before
 // it turns to the others: the blocks of a launch start some microseconds apart, and a
 // second block on one SM would take the groups of SMs whose blocks are about to start
-// (groups of a short list then piled up on a few SMs: 167 to 220 ms for the same call).
+// (groups of a short list then piled up on a few SMs: 166 to 220 ms for the same call).
 // SM s serves list (s + redo_shift) mod L: launches that run side by side (batches)
 // shift their lists, or the longest groups of all of them would meet on the first SMs.
 // Without one (a call that must not touch the shared

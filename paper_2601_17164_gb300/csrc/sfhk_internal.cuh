@@ -208,7 +208,6 @@ constexpr double kWarpsDt = 1e150;
 // scratch, up to the longest call they take
 int64_t fp64_limit(int pot, int sms);
 cudaError_t launch_fp64(const FieldDev& f, const TargetDev& t, const TrajArgs& a, cudaStream_t s);
-int64_t redo_blocks(int64_t n);
 // The high-precision pass over an escalation list: esc_precision 0 FP64 (the split
 // kernel where it applies: planar form, atomic bins), 1 double-float (planar form;
 // FP64 in the 3D form), 2 FP64 with one thread per trajectory.
